@@ -53,6 +53,7 @@ struct hpt_batch_s {
   uint8_t* d_chunks = nullptr;
   hpt::MixedSys* d_tab = nullptr;
   hpt::Fp64Sys* d_f64 = nullptr;
+  bool fixed = true;              // every system has the fixed-point FP64 form
   int32_t* d_sys_n = nullptr;
   int32_t* d_order = nullptr;
   int32_t* d_err = nullptr;
@@ -475,7 +476,7 @@ hpt_status track_impl(hpt_batch_s* b, const int64_t* paths, const void* y0, cons
       const int sh = bk < 2 ? bk : 2;   // FP64: n <= 8, <= 16, <= 32 lane groups
       // evaluation sized for the bucket's variables (n <= 8, 16, 24, 32)
       const int esh = bk < 2 ? bk : (bk == 2 ? kEval24 : 2);
-      e = launch_eval_fp64_map(esh, b->d_f64, q.cap_bucket[bk], x_out, nullptr, pm, d + q.o_ext, st);
+      e = launch_eval_fp64_map(esh, b->d_f64, b->fixed, q.cap_bucket[bk], x_out, nullptr, pm, d + q.o_ext, st);
       if (e == cudaSuccess)
         e = launch_newton_map(sh, q.cap_bucket[bk], d + q.o_ext, x_out, done, last, prm.polish_tol, pm, st);
     }
@@ -586,7 +587,10 @@ hpt_status hpt_batch_create(int32_t nsys, const hpt_system* systems, hpt_batch* 
   if (e == cudaSuccess) e = cudaMalloc(&b->d_tab, sizeof(MixedSys) * nsys);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_tab, tab.data(), sizeof(MixedSys) * nsys, cudaMemcpyHostToDevice);
   std::vector<Fp64Sys> f64(nsys);
-  for (int s = 0; s < nsys; ++s) f64[s] = fp64_sys_of(systems[s]);
+  for (int s = 0; s < nsys; ++s) {
+    f64[s] = fp64_sys_of(systems[s]);
+    b->fixed = b->fixed && f64[s].mono;
+  }
   if (e == cudaSuccess) e = cudaMalloc(&b->d_f64, sizeof(Fp64Sys) * nsys);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_f64, f64.data(), sizeof(Fp64Sys) * nsys, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_sys_n, 4 * nsys);

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "hpt_fx.cuh"
 #include "hpt_internal.h"
 
 namespace hpt {
@@ -404,6 +405,39 @@ static hpt_status upload_constants(hpt_system s, const int32_t* ex) {
   CUU(cudaMemcpy(s->d_off, s->off.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
   CUU(cudaMemcpy(s->d_ahat, ahat.data(), ahat.size() * sizeof(double), cudaMemcpyHostToDevice));
   CUU(cudaMemcpy(s->d_b, b.data(), b.size() * sizeof(double), cudaMemcpyHostToDevice));
+  // the fixed-point form, when every exponent is within its range
+  bool fixed = true;
+  for (int i = 0; i < M && fixed; ++i) {
+    int64_t s1 = 0;
+    for (int j = 0; j < nv; ++j) s1 += std::abs((int64_t)ex[(size_t)i * nv + j]);
+    fixed = s1 <= kFxSum && s->texp[i] <= kFxTexp && s->texp[i] >= -kFxTexp;
+  }
+  if (fixed) {
+    std::vector<FxMono> mono(M);
+    std::vector<FxEnt> ent;
+    for (int i = 0; i < M; ++i) {
+      FxMono& m = mono[i];
+      m.e = (int32_t)s->texp[i];
+      m.eD = (double)s->texp[i] / (double)s->D;
+      m.ef = (float)m.e;
+      fx::Log lg;
+      const bool nonzero = fx::log_of(coeffs[2 * i], coeffs[2 * i + 1], lg);
+      m.lc = lg.l;
+      m.turn = lg.turn;
+      m.lcf = nonzero ? lg.lf : -INFINITY;
+      m.pad_ = 0;
+      m.ent = (int32_t)ent.size();
+      for (int j = 0; j < nv; ++j) {
+        const int32_t a = ex[(size_t)i * nv + j];
+        if (a) ent.push_back(FxEnt{(double)a, a, j});
+      }
+      m.nnz = (int32_t)ent.size() - m.ent;
+    }
+    CUU(cudaMalloc(&s->d_mono, mono.size() * sizeof(FxMono)));
+    CUU(cudaMemcpy(s->d_mono, mono.data(), mono.size() * sizeof(FxMono), cudaMemcpyHostToDevice));
+    CUU(cudaMalloc(&s->d_ent, (ent.size() + 1) * sizeof(FxEnt)));   // a system of constants has none
+    if (!ent.empty()) CUU(cudaMemcpy(s->d_ent, ent.data(), ent.size() * sizeof(FxEnt), cudaMemcpyHostToDevice));
+  }
   if (s->prec != HPT_MIXED) return HPT_OK;
 
   MixedLayout& ml = s->ml;
@@ -1043,6 +1077,8 @@ hpt_status hpt_destroy(hpt_system s) {
   cudaFree(s->d_off);
   cudaFree(s->d_ahat);
   cudaFree(s->d_b);
+  cudaFree(s->d_mono);
+  cudaFree(s->d_ent);
   cudaFree(s->d_chunks);
   cudaFree(s->d_err);
   cudaFree(s->d_scratch);

@@ -62,6 +62,26 @@ struct MixedSys {
   int64_t chunk_off;   // byte offset of the system's constant images
 };
 
+// Fixed-point FP64 evaluation (hpt_eval64.cu): one record per monomial and one
+// per nonzero exponent.  It takes the systems whose monomials have sum |a_j|
+// <= kFxSum (the FP32 copy of an exponent sum then decides its integer part)
+// and |e| <= kFxTexp.
+constexpr int64_t kFxSum = 1024;
+constexpr int64_t kFxTexp = 0x7fffffff;
+struct __align__(16) FxMono {
+  int64_t lc;       // log2|c| modulo 16, Q60
+  uint64_t turn;    // arg c / (2 pi), Q64
+  double eD;        // e / D
+  int32_t e;
+  int32_t ent, nnz; // its nonzero exponents
+  float lcf, ef;    // log2|c| (-inf for c = 0), e
+  int32_t pad_;
+};
+struct __align__(16) FxEnt {
+  double ad;        // the exponent as a double
+  int32_t a, j;     // the exponent and its variable
+};
+
 // One system's FP64 constants as the FP64 evaluation kernel reads them: n
 // equations in nv variables (nv = n, or n + 1 in the projective form).
 struct Fp64Sys {
@@ -70,6 +90,9 @@ struct Fp64Sys {
   const int32_t* off;
   const double* ahat;
   const double2* b;
+  const FxMono* mono;   // null: exponents beyond the fixed point's range
+  const FxEnt* ent;
+  double D;             // denominator of the t-exponents
 };
 
 // Whether a system's coefficient GEMM takes the grouped form, two MMAs per
@@ -172,6 +195,8 @@ struct hpt_system_s {
   int32_t* d_off = nullptr;
   double* d_ahat = nullptr;          // M x (n+1): a_{k,i} and e/D
   double* d_b = nullptr;             // M x (n+2) complex: B_k columns
+  hpt::FxMono* d_mono = nullptr;     // fixed-point form (null: out of its range)
+  hpt::FxEnt* d_ent = nullptr;
   // device constants, mixed form
   hpt::MixedLayout ml;
   uint8_t* d_chunks = nullptr;       // n x chunk_bytes
@@ -224,9 +249,9 @@ Fp64Sys fp64_sys_of(const hpt_system s);
 // The same over the position range [*pm.pos_begin, *pm.npos) of a map whose
 // systems all have shape_of(n) == shape (tab: per-system constants), or with
 // shape kEval24 all n <= 24; cap bounds the range's length.  Writes the
-// extended Jacobian (FP64) only.
+// extended Jacobian (FP64) only.  fixed: every system has the fixed-point form.
 constexpr int kEval24 = 4;
-cudaError_t launch_eval_fp64_map(int shape, const Fp64Sys* tab, int64_t cap, const void* y, const double* tau,
+cudaError_t launch_eval_fp64_map(int shape, const Fp64Sys* tab, bool fixed, int64_t cap, const void* y, const double* tau,
                                  const PathMap& pm, void* ext, cudaStream_t st);
 
 // Mixed tensor-core evaluation, complex64 in and out.
