@@ -353,7 +353,7 @@ cudaError_t launch_fx(const Fp64Sys& f, int nvs, int neq, int64_t p, const doubl
   const int64_t tiles = (p + 31) / 32;
   if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
   const int smem = fx_smem(nvs, Hy != nullptr);
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {   // static shared memory (5 KB) counts towards the default 48 KB too
     cudaError_t e = cudaFuncSetAttribute(eval_fx_kernel<MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, fx_smem(kMaxN, true));
     if (e != cudaSuccess) return e;
   }
