@@ -307,10 +307,10 @@ hpt_paths offset_paths(const hpt_paths& S, int64_t q0, int nv, size_t cs);
 int solve_shape_of(int n);
 constexpr int kShape8x3 = 3;   // FP32 solve only: 8 lanes x 3 rows per path, n <= 24
 // FP64 Newton polish update over the position range [*pm.pos_begin,
-// *pm.npos) of a map (shape as above; cap bounds the range's length); x is
+// *pm.npos) of a map (systems of n <= nbound; cap bounds the range's length); x is
 // complex128 at pm.vofs, done and last (the previous relative correction)
 // per path.
-cudaError_t launch_newton_map(int shape, int64_t cap, const void* ext, void* x, int32_t* done, float* last,
+cudaError_t launch_newton_map(int nbound, int64_t cap, const void* ext, void* x, int32_t* done, float* last,
                               double tol, const PathMap& pm, cudaStream_t st);
 cudaError_t launch_solve_fp32_shape(int shape, const StepArgs& a, cudaStream_t st);
 cudaError_t launch_redo_fp64_shape(int shape, const StepArgs& a, cudaStream_t st);

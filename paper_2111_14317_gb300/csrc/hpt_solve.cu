@@ -22,8 +22,10 @@
 
 #include <algorithm>
 
-#include "hpt_internal.h"
 #include "hpt_cx.cuh"
+#include "hpt_fx.cuh"
+#include "hpt_internal.h"
+#include "hpt_lu64.cuh"
 
 namespace hpt {
 namespace {
@@ -357,6 +359,45 @@ __device__ __forceinline__ void load_step_state(int n, int64_t path, size_t vbas
   Q.streak = S.streak[path];
 }
 
+// Largest modulus over a group's entries: the largest square first (bit
+// patterns of non-negative doubles compare as integers) and one square root,
+// since each hypot costs some 25 instructions of the FP64 pipe; squares
+// outside [1e-280, 1e280] take the hypots.  NaN entries are the caller's to
+// find.
+template <int G, int R>
+__device__ __forceinline__ double group_max_abs(const cx<double> (&v)[R], int n, unsigned gmask) {
+  const int lane = threadIdx.x & (G - 1);
+  unsigned long long m2 = 0;
+#pragma unroll
+  for (int s = 0; s < R; ++s)
+    if (lane + G * s < n) m2 = max(m2, (unsigned long long)__double_as_longlong(abs2(v[s])));
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) m2 = max(m2, __shfl_xor_sync(gmask, m2, o, G));
+  const double sq = __longlong_as_double((long long)m2);
+  if (m2 == 0 || (sq > 1e-280 && sq < 1e280)) return sqrt(sq);
+  double m = 0.0;
+#pragma unroll
+  for (int s = 0; s < R; ++s)
+    if (lane + G * s < n) m = fmax(m, cabs_t(v[s]));
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(gmask, m, o, G));
+  return m;
+}
+
+// Whether a modulus lies outside (1/bound, bound) (or is NaN); FP64 by
+// squares where these cannot leave the range.
+template <typename TS>
+__device__ __forceinline__ bool outside_bound(cx<TS> v, double bound) {
+  if constexpr (sizeof(TS) == 8) {
+    if (bound < 1e140) {
+      const double m2 = abs2(v), b2 = bound * bound;
+      return !(m2 < b2) || !(m2 * b2 > 1.0);
+    }
+  }
+  const TS m = cabs_t(v);
+  return !(m < (TS)bound) || !(m > (TS)(1.0 / bound));
+}
+
 template <typename TS, int G, int R>
 __device__ __forceinline__ void update_path(int n, int64_t path, size_t vbase, int32_t status, bool ok,
                                             const cx<TS> (&wE)[R], const cx<TS> (&wN)[R], const hpt_paths& S,
@@ -379,15 +420,22 @@ __device__ __forceinline__ void update_path(int n, int64_t path, size_t vbase, i
     xN[s] = cmul(y[s], wN[s]);
     if (mine) {
       solfin = solfin && finite(xE[s]) && finite(xN[s]);
-      ny = t_max(ny, cabs_t(y[s]));
-      nd = t_max(nd, cabs_t(xN[s]));
+      if constexpr (sizeof(TS) == 4) {
+        ny = t_max(ny, cabs_t(y[s]));
+        nd = t_max(nd, cabs_t(xN[s]));
+      }
     }
   }
   solfin = (__ballot_sync(gmask, solfin) & gmask) == gmask;
+  if constexpr (sizeof(TS) == 4) {
 #pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) {
-    ny = t_max(ny, __shfl_xor_sync(gmask, ny, o, G));
-    nd = t_max(nd, __shfl_xor_sync(gmask, nd, o, G));
+    for (int o = G / 2; o > 0; o >>= 1) {
+      ny = t_max(ny, __shfl_xor_sync(gmask, ny, o, G));
+      nd = t_max(nd, __shfl_xor_sync(gmask, nd, o, G));
+    }
+  } else {
+    ny = group_max_abs<G, R>(y, n, gmask);
+    nd = group_max_abs<G, R>(xN, n, gmask);
   }
   const bool bad = !(ok && solfin);
   double tau = Q.tau, dtau = Q.dtau, tauacc = Q.tauacc;
@@ -418,10 +466,7 @@ __device__ __forceinline__ void update_path(int n, int64_t path, size_t vbase, i
       bool div = false;
 #pragma unroll
       for (int s = 0; s < R; ++s) {
-        if (lane + G * s < n) {
-          const TS m = cabs_t(yacc[s]);
-          div = div || !(m < (TS)prm.div_bound) || !(m > (TS)(1.0 / prm.div_bound));
-        }
+        if (lane + G * s < n) div = div || outside_bound<TS>(yacc[s], prm.div_bound);
       }
       div = (__ballot_sync(gmask, div) & gmask) != 0u;
       if (div) {
@@ -977,60 +1022,89 @@ redo_fp64_kernel(int n0, const void* __restrict__ ext, hpt_paths S, hpt_params p
   }
 }
 
+// One FP64 Euler-Newton step per ACTIVE path: consolidated solve in shared
+// memory (lu64_solve), then the step control.  128 / G consecutive paths per
+// block.
+template <int G, int R>
+__global__ void __launch_bounds__(kLuThreads)
+step_fp64_kernel(int n, int64_t p, const double2* __restrict__ ext, hpt_paths S, hpt_params prm) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int P = lu64_paths<G>();
+  const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
+  const int64_t q0 = (int64_t)blockIdx.x * P;
+  const int stride = lu64_entries(n), cstride = 4 * lu64_col_entries(n);
+  double2* mats = (double2*)smem;
+  {
+    const int i = threadIdx.x % P;
+    const int64_t qi = q0 + i;
+    lu64_stage<G>(n, n, ext, qi, qi < p && S.status[qi] == HPT_PATH_ACTIVE, mats + i * stride, false);
+  }
+  const int64_t path = q0 + g;
+  const int32_t status = path < p ? S.status[path] : -1;
+  const bool valid = status == HPT_PATH_ACTIVE;
+  __syncthreads();
+  if (!__any_sync(0xffffffffu, valid)) return;   // warp-uniform exit
+  double2* A = mats + g * stride;
+  int* colx = (int*)(mats + P * stride) + g * cstride;
+  const bool ok = lu64_solve<G>(n, A, colx, -1);
+  if (!valid) return;   // group-uniform; only group-masked shuffles below
+  cx<double> xE[R], xN[R];
+#pragma unroll
+  for (int s = 0; s < R; ++s) {
+    const int c = lane + G * s;
+    xE[s] = c < n ? lu64_x(n, A, colx, c, 0) : mk<double>(0, 0);
+    xN[s] = c < n ? lu64_x(n, A, colx, c, 1) : mk<double>(0, 0);
+  }
+  update_path<double, G, R>(n, path, (size_t)path * n, status, ok, xE, xN, S, prm);
+}
+
 // Newton polish update at t = 1 (FP64): x += dN until the error left is below
 // tol: |dN|/max(1,|x|) <= tol, or, once the corrections shrink quadratically,
 // the error after this update, about r_k^3 / r_{k-1}^2 for the relative
 // corrections r of the last two iterations (last[] keeps r_{k-1}; 0: none).
-// MAP: positions [*pm.pos_begin, *pm.npos) of a position map (a warp's
-// positions lie in one tile, so n is warp-uniform); otherwise the p paths of
+// MAP: positions [*pm.pos_begin, *pm.npos) of a position map (a block's
+// positions lie in one tile, so n is block-uniform); otherwise the p paths of
 // one system.
 template <int G, int R, bool MAP>
-__global__ void __launch_bounds__(kSolveThreads)
-newton_kernel(int n0, int64_t p, const void* __restrict__ ext, double2* __restrict__ x,
+__global__ void __launch_bounds__(kLuThreads)
+newton_kernel(int n0, int64_t p, const double2* __restrict__ ext, double2* __restrict__ x,
               int32_t* __restrict__ done, float* __restrict__ last, double tol, PathMap pm) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & (G - 1);
-  const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G + (MAP ? (int64_t)*pm.pos_begin : 0);
+  constexpr int P = lu64_paths<G>();
+  const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
+  const int64_t q0 = (int64_t)blockIdx.x * P + (MAP ? (int64_t)*pm.pos_begin : 0);
   const int64_t end = MAP ? (int64_t)*pm.npos : p;
-  const bool in = q < end;
-  const int64_t path = in ? (MAP ? pm.list[q] : q) : -1;
-  const bool valid = path >= 0 && done[path] == 0;
-  unsigned char* sm = smem + (threadIdx.x / G) * GroupSmem<double, G * R>::bytes;
-  if (G == 32) {   // block-uniform: stage the block's four positions
-    const int64_t q0 = q - (threadIdx.x >> 5);
-    if (q0 >= end) return;   // the whole block (end is a multiple of 4)
-    const int n = MAP ? pm.sys_n[pm.tile_sys[q0 >> 7]] : n0;
-    const int64_t qi = q0 + (threadIdx.x & 3);
-    const int64_t pi = qi < end ? (MAP ? pm.list[qi] : qi) : -1;
-    stage_block_rows<double>(n, MAP ? pm.nmax : n, ext, q0, pi >= 0 && done[pi] == 0, smem,
-                             GroupSmem<double, G * R>::bytes);
-    __syncthreads();
+  if (q0 >= end) return;
+  const int n = MAP ? pm.sys_n[pm.tile_sys[q0 >> 7]] : n0;
+  const int stride = lu64_entries(n), cstride = 4 * lu64_col_entries(n);
+  double2* mats = (double2*)smem;
+  {
+    const int i = threadIdx.x % P;
+    const int64_t qi = q0 + i, pi = qi < end ? (MAP ? pm.list[qi] : qi) : -1;
+    lu64_stage<G>(n, MAP ? pm.nmax : n, ext, qi, pi >= 0 && done[pi] == 0, mats + i * stride, false);
   }
+  const int64_t q = q0 + g;
+  const int64_t path = q < end ? (MAP ? pm.list[q] : q) : -1;
+  const bool valid = path >= 0 && done[path] == 0;
+  __syncthreads();
   if (!__any_sync(0xffffffffu, valid)) return;
-  const int n = MAP ? pm.sys_n[pm.tile_sys[q >> 7]] : n0;
-  const size_t vbase = MAP ? (valid ? (size_t)pm.vofs[path] : 0) : (size_t)path * n;
-  PathRows<double, G, R> P;
-  bool fin;
-  if constexpr (G == 32) fin = load_rows_staged<double, double>(n, sm, valid, P);
-  else fin = load_rows<double, double, G, R>(n, MAP ? pm.nmax : n, ext, q, vbase, valid, false, nullptr, P);
-  cx<double> xE[R], xN[R];
-  double cond;
-  const bool ok = group_solve<double, G, R>(n, P, xE, xN, cond, sm) && fin;
+  double2* A = mats + g * stride;
+  int* colx = (int*)(mats + P * stride) + g * cstride;
+  const bool ok = lu64_solve<G>(n, A, colx, -1);
   if (!valid) return;
+  const size_t vbase = MAP ? (size_t)pm.vofs[path] : (size_t)path * n;
   const unsigned gmask = group_mask<G>();
   bool sfin = true;
-  double ny = 0.0, nd = 0.0;
-  cx<double> y[R];
+  cx<double> y[R], xN[R];
 #pragma unroll
   for (int s = 0; s < R; ++s) {
     const int j = lane + G * s;
-    y[s] = j < n ? ld<double>(x, vbase + j) : mk<double>(0, 0);
-    xN[s] = cmul(y[s], xN[s]);   // D_z H in the scratch: the correction is x * w
+    y[s] = xN[s] = mk<double>(0, 0);
     if (j < n) {
+      y[s] = ld<double>(x, vbase + j);
+      xN[s] = cmul(y[s], lu64_x(n, A, colx, j, 1));   // D_z H in the scratch: the correction is x * w
       sfin = sfin && finite(xN[s]);
       y[s] = mk<double>(y[s].x + xN[s].x, y[s].y + xN[s].y);
-      ny = fmax(ny, cabs_t(y[s]));
-      nd = fmax(nd, cabs_t(xN[s]));
     }
   }
   sfin = (__ballot_sync(gmask, sfin) & gmask) == gmask;
@@ -1038,11 +1112,7 @@ newton_kernel(int n0, int64_t p, const void* __restrict__ ext, double2* __restri
     if (lane == 0) done[path] = 2;
     return;
   }
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) {
-    ny = fmax(ny, __shfl_xor_sync(gmask, ny, o, G));
-    nd = fmax(nd, __shfl_xor_sync(gmask, nd, o, G));
-  }
+  const double ny = group_max_abs<G, R>(y, n, gmask), nd = group_max_abs<G, R>(xN, n, gmask);
 #pragma unroll
   for (int s = 0; s < R; ++s) {
     const int j = lane + G * s;
@@ -1058,65 +1128,91 @@ newton_kernel(int n0, int64_t p, const void* __restrict__ ext, double2* __restri
 
 // Adjoint, part 1: per solution, lambda from J^H lambda = gx (J from the
 // extended Jacobian at t = 1), then contrib[q][i] = -lambda_k conj(x^{a_i})
-// for every monomial i of equation k (monomials by exp of <a, log x>).
+// for every monomial i of equation k.  The monomials of a solution are dealt
+// to its G lanes (consecutive contributions, whole sectors) and come from the
+// fixed-point logarithm and exponential (hpt_fx.cuh), which leave the FP64
+// pipe four operations a monomial; systems beyond their range (no mono)
+// take exp of <a, log x> in FP64.
 template <int G, int R>
-__global__ void __launch_bounds__(kSolveThreads)
-adjoint_kernel(int n, int64_t p, const int32_t* __restrict__ msz, const int32_t* __restrict__ off,
-               const double* __restrict__ ahat, int M, const void* __restrict__ ext,
-               const double2* __restrict__ x, const double2* __restrict__ gx,
-               double2* __restrict__ contrib) {
+__global__ void __launch_bounds__(kLuThreads)
+adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, const double2* __restrict__ x,
+               const double2* __restrict__ gx, double2* __restrict__ contrib) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double2 zsh[kSolveThreads / G][G * R];
-  const int lane = threadIdx.x & (G - 1);
-  const int grp = threadIdx.x / G;
-  const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  constexpr int P = lu64_paths<G>();
+  __shared__ ulonglong2 zsh[P][G * R];
+  __shared__ float lfs[P][G * R];
+  const int n = sys.n;
+  const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
+  const int64_t q0 = (int64_t)blockIdx.x * P;
+  const int stride = lu64_entries(n), cstride = 4 * lu64_col_entries(n);
+  double2* mats = (double2*)smem;
+  {
+    const int i = threadIdx.x % P;
+    lu64_stage<G>(n, n, ext, q0 + i, q0 + i < p, mats + i * stride, true);
+  }
+  const int64_t path = q0 + g;
   const bool valid = path < p;
-  PathRows<double, G, R> P;
-  const bool fin = load_rows<double, double, G, R>(n, n, ext, path, (size_t)path * n, valid, true, gx, P);
+  double2* A = mats + g * stride;
+  int* colx = (int*)(mats + P * stride) + g * cstride;
   // D_z H = H_y diag(x) in the scratch: H_y^H lambda = g becomes
   // (D_z H)^H lambda = conj(x) g
 #pragma unroll
   for (int s = 0; s < R; ++s) {
     const int r = lane + G * s;
     if (valid && r < n) {
-      const double2 v = x[(size_t)path * n + r];
-      P.bE[s] = cmul(mk<double>(v.x, -v.y), P.bE[s]);
-    }
-  }
-  cx<double> lam[R], dummy[R];
-  double cond;
-  const bool ok =
-      group_solve<double, G, R>(n, P, lam, dummy, cond, smem + grp * GroupSmem<double, G * R>::bytes) && fin;
-#pragma unroll
-  for (int s = 0; s < R; ++s) {
-    const int j = lane + G * s;
-    if (valid && j < n) {
-      const double2 v = x[(size_t)path * n + j];
-      zsh[grp][j] = make_double2(log(hypot(v.x, v.y)), atan2(v.y, v.x));
+      const double2 v = x[(size_t)path * n + r], w = gx[(size_t)path * n + r];
+      const cx<double> b = cmul(mk<double>(v.x, -v.y), mk<double>(w.x, w.y));
+      A[r * (n + 2) + n] = make_double2(b.x, b.y);
+      A[r * (n + 2) + n + 1] = make_double2(0.0, 0.0);
+      if (sys.mono) {
+        fx::Log lg;
+        fx::log_of(v.x, v.y, lg);
+        zsh[g][r] = make_ulonglong2((unsigned long long)lg.l, lg.turn);
+        lfs[g][r] = lg.lf;
+      } else {
+        zsh[g][r] = make_ulonglong2((unsigned long long)__double_as_longlong(log(hypot(v.x, v.y))),
+                                    (unsigned long long)__double_as_longlong(atan2(v.y, v.x)));
+      }
     }
   }
   __syncthreads();
+  if (!__any_sync(0xffffffffu, valid)) return;
+  const bool ok = lu64_solve<G>(n, A, colx, 1);
   if (!valid) return;
-#pragma unroll
-  for (int s = 0; s < R; ++s) {
-    const int k = lane + G * s;
-    if (k >= n) continue;
-    for (int i = off[k]; i < off[k] + msz[k]; ++i) {
-      const double* ai = ahat + (size_t)i * (n + 1);
+  const fx::Tables& T = fx::tables();
+  for (int k = 0, i = lane; i < M; i += G) {
+    while (i >= sys.off[k] + sys.msz[k]) ++k;
+    double mr, mi;
+    if (sys.mono) {
+      const FxMono m = sys.mono[i];
+      int64_t W = 0;
+      uint64_t th = 0;
+      float wf = 0.f;
+      for (int t = 0; t < m.nnz; ++t) {
+        const int a = sys.ent[m.ent + t].a, j = sys.ent[m.ent + t].j;
+        const ulonglong2 z = zsh[g][j];
+        W += (int64_t)a * (int64_t)z.x;
+        th += (uint64_t)((int64_t)a * (int64_t)z.y);
+        wf = fmaf((float)a, lfs[g][j], wf);
+      }
+      fx::exp_of(W, th, wf, T.exp1, T.exp2, T.cs1, T.cs2, mr, mi);
+    } else {
+      const double* ai = sys.ahat + (size_t)i * (n + 1);
       double wr = 0.0, wi = 0.0;
       for (int j = 0; j < n; ++j) {
-        wr = fma(ai[j], zsh[grp][j].x, wr);
-        wi = fma(ai[j], zsh[grp][j].y, wi);
+        wr = fma(ai[j], __longlong_as_double((long long)zsh[g][j].x), wr);
+        wi = fma(ai[j], __longlong_as_double((long long)zsh[g][j].y), wi);
       }
-      double sn, cs;
-      sincos(wi, &sn, &cs);
+      sincos(wi, &mi, &mr);
       const double m = exp(wr);
-      // -lambda_k * conj(m (cs + i sn))
-      const double mr = m * cs, mi = -m * sn;
-      double2 v = make_double2(-(lam[s].x * mr - lam[s].y * mi), -(lam[s].x * mi + lam[s].y * mr));
-      if (!ok) v = make_double2(NAN, NAN);
-      contrib[(size_t)path * M + i] = v;
+      mr *= m;
+      mi *= m;
     }
+    // -lambda_k conj(x^a)
+    const cx<double> lam = lu64_x(n, A, colx, k, 0);
+    double2 v = make_double2(-(lam.x * mr + lam.y * mi), lam.x * mi - lam.y * mr);
+    if (!ok) v = make_double2(NAN, NAN);
+    contrib[(size_t)path * M + i] = v;
   }
 }
 
@@ -1302,33 +1398,61 @@ cudaError_t launch_redo_shape(const StepArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// The FP64 solves: (G, R) = (8, 1) for n <= 8, (8, 2) for n <= 16, (16, 2) for
+// n <= 32 where the paths fill the chip; 32 lanes a path where fewer than
+// kLuWarps warps would be in flight: a path's chain is then shorter (the
+// lanes that a step's entries do not fill cost nothing on an idle pipe).
+// Every shape gives the same bits.
+constexpr int64_t kLuWarps = 152 * 4 * 2;
+inline int lu_shape(int n, int64_t p) {
+  const int G = n <= 16 ? 8 : 16;
+  if (p * G < 32 * kLuWarps) return 3;
+  return n <= 8 ? 0 : (n <= 16 ? 1 : 2);
+}
+
+template <int G, int R>
+cudaError_t launch_step64_shape(const StepArgs& a, cudaStream_t st) {
+  const int smem = lu64_smem<G>(a.n);
+  cudaError_t e = set_smem(step_fp64_kernel<G, R>, lu64_smem<G>(G * R));
+  if (e != cudaSuccess) return e;
+  step_fp64_kernel<G, R><<<blocks_for(a.p, lu64_paths<G>()), kLuThreads, smem, st>>>(
+      a.n, a.p, (const double2*)a.ext, a.st, a.prm);
+  return cudaGetLastError();
+}
+
 template <int G, int R>
 cudaError_t launch_newton_shape(int n, int64_t p, const void* ext, void* x, int32_t* done, float* last,
                                 double tol, const PathMap* pm, cudaStream_t st) {
-  const int smem = (kSolveThreads / G) * GroupSmem<double, G * R>::bytes;
-  if (pm) {
-    cudaError_t e = set_smem(newton_kernel<G, R, true>, smem);
-    if (e != cudaSuccess) return e;
-    newton_kernel<G, R, true><<<blocks_for(p * G, kSolveThreads), kSolveThreads, smem, st>>>(
-        n, p, ext, (double2*)x, done, last, tol, *pm);
-    return cudaGetLastError();
-  }
-  cudaError_t e = set_smem(newton_kernel<G, R, false>, smem);
+  const int smem = lu64_smem<G>(n);   // map: n bounds the range's systems
+  cudaError_t e = pm ? set_smem(newton_kernel<G, R, true>, lu64_smem<G>(G * R))
+                     : set_smem(newton_kernel<G, R, false>, lu64_smem<G>(G * R));
   if (e != cudaSuccess) return e;
-  newton_kernel<G, R, false><<<blocks_for(p * G, kSolveThreads), kSolveThreads, smem, st>>>(
-      n, p, ext, (double2*)x, done, last, tol, PathMap());
+  const unsigned nb = blocks_for(p, lu64_paths<G>());
+  if (pm)
+    newton_kernel<G, R, true><<<nb, kLuThreads, smem, st>>>(n, p, (const double2*)ext, (double2*)x, done, last, tol, *pm);
+  else
+    newton_kernel<G, R, false><<<nb, kLuThreads, smem, st>>>(n, p, (const double2*)ext, (double2*)x, done, last, tol,
+                                                             PathMap());
   return cudaGetLastError();
+}
+
+cudaError_t launch_newton(int n, int64_t p, const void* ext, void* x, int32_t* done, float* last, double tol,
+                          const PathMap* pm, cudaStream_t st) {
+  const int sh = lu_shape(n, p);
+  return sh == 0 ? launch_newton_shape<8, 1>(n, p, ext, x, done, last, tol, pm, st)
+       : sh == 1 ? launch_newton_shape<8, 2>(n, p, ext, x, done, last, tol, pm, st)
+       : sh == 2 ? launch_newton_shape<16, 2>(n, p, ext, x, done, last, tol, pm, st)
+                 : launch_newton_shape<32, 1>(n, p, ext, x, done, last, tol, pm, st);
 }
 
 template <int G, int R>
 cudaError_t launch_adjoint_shape(hpt_system s, int64_t p, const void* ext, const void* x, const void* gx,
                                  void* contrib, cudaStream_t st) {
-  const int smem = (kSolveThreads / G) * GroupSmem<double, G * R>::bytes;
-  cudaError_t e = set_smem(adjoint_kernel<G, R>, smem);
+  const int smem = lu64_smem<G>(s->n);
+  cudaError_t e = set_smem(adjoint_kernel<G, R>, lu64_smem<G>(G * R));
   if (e != cudaSuccess) return e;
-  adjoint_kernel<G, R><<<blocks_for(p * G, kSolveThreads), kSolveThreads, smem, st>>>(
-      s->n, p, s->d_msz, s->d_off, s->d_ahat, s->M, ext, (const double2*)x, (const double2*)gx,
-      (double2*)contrib);
+  adjoint_kernel<G, R><<<blocks_for(p, lu64_paths<G>()), kLuThreads, smem, st>>>(
+      fp64_sys_of(s), p, s->M, (const double2*)ext, (const double2*)x, (const double2*)gx, (double2*)contrib);
   return cudaGetLastError();
 }
 
@@ -1340,9 +1464,11 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
   cudaError_t e;
   if (s->prec == HPT_FP64) {
     int pi = prof_begin(s, "solve_update_fp64", st);
-    e = shape == 0 ? launch_solve_shape<double, 8, 1>(a, nullptr, nullptr, st)
-      : shape == 1 ? launch_solve_shape<double, 8, 2>(a, nullptr, nullptr, st)
-                   : launch_solve_shape<double, 32, 1>(a, nullptr, nullptr, st);
+    const int sh = lu_shape(a.n, a.p);
+    e = sh == 0 ? launch_step64_shape<8, 1>(a, st)
+      : sh == 1 ? launch_step64_shape<8, 2>(a, st)
+      : sh == 2 ? launch_step64_shape<16, 2>(a, st)
+                : launch_step64_shape<32, 1>(a, st);
     prof_end(s, pi, st);
     return e;
   }
@@ -1371,13 +1497,11 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
 
 int solve_shape_of(int n) { return shape_of(n); }
 
-cudaError_t launch_newton_map(int shape, int64_t cap, const void* ext, void* x, int32_t* done, float* last,
+cudaError_t launch_newton_map(int nbound, int64_t cap, const void* ext, void* x, int32_t* done, float* last,
                               double tol, const PathMap& pm, cudaStream_t st) {
   if (cap <= 0) return cudaSuccess;
   if (!pm.list || !pm.tile_sys || !pm.sys_n || !pm.vofs || !pm.npos || !pm.pos_begin) return cudaErrorInvalidValue;
-  return shape == 0 ? launch_newton_shape<8, 1>(0, cap, ext, x, done, last, tol, &pm, st)
-       : shape == 1 ? launch_newton_shape<8, 2>(0, cap, ext, x, done, last, tol, &pm, st)
-                    : launch_newton_shape<32, 1>(0, cap, ext, x, done, last, tol, &pm, st);
+  return launch_newton(nbound, cap, ext, x, done, last, tol, &pm, st);
 }
 
 cudaError_t launch_solve_fp32_shape(int shape, const StepArgs& a, cudaStream_t st) {
@@ -1398,11 +1522,8 @@ cudaError_t launch_redo_fp64_shape(int shape, const StepArgs& a, cudaStream_t st
 cudaError_t launch_newton_update(hpt_system s, int64_t p, const void* ext, void* x, int32_t* done,
                                  float* last, double tol, cudaStream_t st) {
   if (p <= 0) return cudaSuccess;
-  const int shape = shape_of(s->n);
   int pi = prof_begin(s, "newton_fp64", st);
-  cudaError_t e = shape == 0 ? launch_newton_shape<8, 1>(s->n, p, ext, x, done, last, tol, nullptr, st)
-                : shape == 1 ? launch_newton_shape<8, 2>(s->n, p, ext, x, done, last, tol, nullptr, st)
-                             : launch_newton_shape<32, 1>(s->n, p, ext, x, done, last, tol, nullptr, st);
+  cudaError_t e = launch_newton(s->n, p, ext, x, done, last, tol, nullptr, st);
   prof_end(s, pi, st);
   return e;
 }
@@ -1412,10 +1533,11 @@ size_t adjoint_part_bytes(int M) { return (size_t)kAdjRowBlocks * M * 16; }
 cudaError_t launch_adjoint(hpt_system s, int64_t p, const void* ext, const void* x, const void* gx,
                            void* partial, void* part, void* gc, cudaStream_t st) {
   if (p <= 0) return cudaSuccess;
-  const int shape = shape_of(s->n);
+  const int shape = lu_shape(s->n, p);
   int pi = prof_begin(s, "adjoint_fp64", st);
   cudaError_t e = shape == 0 ? launch_adjoint_shape<8, 1>(s, p, ext, x, gx, partial, st)
                 : shape == 1 ? launch_adjoint_shape<8, 2>(s, p, ext, x, gx, partial, st)
+                : shape == 2 ? launch_adjoint_shape<16, 2>(s, p, ext, x, gx, partial, st)
                              : launch_adjoint_shape<32, 1>(s, p, ext, x, gx, partial, st);
   prof_end(s, pi, st);
   if (e != cudaSuccess) return e;
