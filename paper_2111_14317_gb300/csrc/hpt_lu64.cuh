@@ -65,21 +65,22 @@ __device__ __forceinline__ double rcp_newton(double v) {
 // of path t % P (P = 128 / G paths, consecutive positions from q0), so that P
 // threads read consecutive addresses of the position-interleaved scratch.
 // conj: the entry (k, u < n) goes to row u, column k, conjugated (the adjoint
-// system); the right-hand sides are then the caller's.
+// system); the right-hand sides are then the caller's.  rows < n: the
+// projective system's equations (its last row is the caller's).
 template <int G>
-__device__ __forceinline__ void lu64_stage(int n, int nmax, const double2* __restrict__ ext, int64_t q, bool act,
+__device__ __forceinline__ void lu64_stage(int rows, int n, int nmax, const double2* __restrict__ ext, int64_t q, bool act,
                                            double2* region, bool conj) {
   if (!act) return;
   const int np2 = n + 2, e0 = threadIdx.x / lu64_paths<G>();
   const double2* src = ext + (size_t)(q >> 7) * (size_t)(nmax * (nmax + 2)) * 128 + (size_t)(q & 127);
   if (nmax == n && !conj) {
-    const int total = n * np2;
+    const int total = rows * np2;
 #pragma unroll 6
     for (int e = e0; e < total; e += G) region[e] = src[(size_t)e * 128];
     return;
   }
   const int w = conj ? n : np2;
-  for (int e = e0; e < n * w; e += G) {
+  for (int e = e0; e < rows * w; e += G) {
     const int k = e / w, u = e - k * w;
     const double2 v = src[((size_t)k * (nmax + 2) + u) * 128];
     if (conj) region[u * np2 + k] = make_double2(v.x, -v.y);
@@ -241,6 +242,18 @@ __device__ __forceinline__ cx<double> lu64_x(int n, const double2* A, const int*
   const double2 v = A[c * (n + 2) + n + b];
   const int k = colx[c];
   return mk<double>(scale_exp(v.x, k), scale_exp(v.y, k));
+}
+
+// The FP64 solves: (G, R) = (8, 1) for n <= 8, (8, 2) for n <= 16, (16, 2) for
+// n <= 32 where the paths fill the chip; 32 lanes a path where fewer than
+// kLuWarps warps would be in flight: a path's chain is then shorter (the
+// lanes that a step's entries do not fill cost nothing on an idle pipe).
+// Every shape gives the same bits.
+constexpr int64_t kLuWarps = 152 * 4 * 2;
+inline int lu_shape(int n, int64_t p) {
+  const int G = n <= 16 ? 8 : 16;
+  if (p * G < 32 * kLuWarps) return 3;
+  return n <= 8 ? 0 : (n <= 16 ? 1 : 2);
 }
 
 }  // namespace

@@ -37,6 +37,7 @@
 
 #include "hpt_cx.cuh"
 #include "hpt_internal.h"
+#include "hpt_lu64.cuh"
 
 namespace hpt {
 namespace {
@@ -69,11 +70,6 @@ __device__ __forceinline__ void ld_pair(const cx<float>* U, int i, cx<float>& g0
   g0 = mk<float>(v.x, v.y);
   g1 = mk<float>(v.z, v.w);
 }
-__device__ __forceinline__ void ld_pair(const cx<double>* U, int i, cx<double>& g0, cx<double>& g1) {
-  g0 = U[i];
-  g1 = U[i + 1];
-}
-
 // Row order.  The rows are factored in index order, and slot s of every lane
 // holds a block of consecutive rows, so that whole slots finish early and are
 // skipped (a warp-uniform test): the first r0 = N - G (R - 1) rows sit in the
@@ -543,6 +539,69 @@ qr_kernel(int n, int nv, int proj, int64_t p, const void* __restrict__ ext, cons
   }
 }
 
+// The FP64 form of the same.  The 2 x 2 reduction of the null space leaves the
+// vectors (dE, 1, 0) and (dN, 0, 1): J's first N columns times dE = -(dH/dtau,
+// 0), times dN = -(H, 0).  So both directions are the solutions of one N x N
+// system, and FP64 takes them from lu64_solve (partial pivoting on the
+// equilibrated rows), N^3/3 complex operations instead of the reflectors' 4/3
+// N^3 on the FP64 pipe that bounds them.  Measured, n = 8 (N = 9), 4,999
+// points: 301 -> 51 us.
+template <int G, int R, bool STEP>
+__global__ void __launch_bounds__(kLuThreads)
+null64_kernel(int n, int nv, int proj, int64_t p, const double2* __restrict__ ext, const double2* __restrict__ yin,
+              double2* __restrict__ dE, double2* __restrict__ dN, int32_t* __restrict__ okout, hpt_paths S,
+              hpt_params prm) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int P = lu64_paths<G>();
+  const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
+  const int64_t q0 = (int64_t)blockIdx.x * P;
+  const int stride = lu64_entries(nv), cstride = 4 * lu64_col_entries(nv);
+  double2* mats = (double2*)smem;
+  {
+    const int i = threadIdx.x % P;
+    const int64_t qi = q0 + i;
+    lu64_stage<G>(n, nv, nv, ext, qi, qi < p && (!STEP || S.status[qi] == HPT_PATH_ACTIVE), mats + i * stride, false);
+  }
+  const int64_t path = q0 + g;
+  const int32_t status = path < p ? (STEP ? S.status[path] : HPT_PATH_ACTIVE) : -1;
+  const bool valid = status == HPT_PATH_ACTIVE;
+  const size_t vbase = valid ? (size_t)path * nv : 0;
+  double2* A = mats + g * stride;
+  int* colx = (int*)(mats + P * stride) + g * cstride;
+  cx<double> y[R];
+#pragma unroll
+  for (int s = 0; s < R; ++s) {
+    const int c = lane + G * s;
+    y[s] = valid && c < nv ? ld<double>(STEP ? S.y : yin, vbase + c) : mk<double>(0, 0);
+    if (proj && c < nv) A[n * (nv + 2) + c] = make_double2(abs2(y[s]), 0.0);   // y^* in log coordinates
+  }
+  if (proj && lane < 2) A[n * (nv + 2) + nv + lane] = make_double2(0.0, 0.0);
+  __syncthreads();
+  if (!__any_sync(0xffffffffu, valid)) return;   // warp-uniform exit
+  const bool ok = lu64_solve<G>(nv, A, colx, -1);
+  if (!valid) return;   // group-uniform; only group-masked shuffles below
+  cx<double> xE[R], xN[R];
+#pragma unroll
+  for (int s = 0; s < R; ++s) {
+    const int j = lane + G * s;
+    xE[s] = j < nv ? cmul(y[s], lu64_x(nv, A, colx, j, 0)) : mk<double>(0, 0);
+    xN[s] = j < nv ? cmul(y[s], lu64_x(nv, A, colx, j, 1)) : mk<double>(0, 0);
+  }
+  if constexpr (STEP) {
+    update_proj<double, G, R>(n, nv, path, vbase, status, ok, xE, xN, S, prm);
+  } else {
+#pragma unroll
+    for (int s = 0; s < R; ++s) {
+      const int j = lane + G * s;
+      if (j < nv) {
+        st<double>(dE, vbase + j, xE[s]);
+        st<double>(dN, vbase + j, xN[s]);
+      }
+    }
+    if (lane == 0) okout[path] = ok ? 1 : 0;
+  }
+}
+
 template <typename T>
 __global__ void paths_init_proj_kernel(int n, int64_t p, const double2* __restrict__ x0, double tau0, double dtau0,
                                        hpt_paths S) {
@@ -618,21 +677,35 @@ cudaError_t launch_qr_shape(hpt_system s, int64_t p, const void* ext, const void
   return cudaGetLastError();
 }
 
-// Shapes by N = nv (CM >= N + 2 columns in registers): (G, R, CM) =
-// (8, 1, 10) for N <= 8, (8, 2, 18) for N <= 16; FP32: (8, 3, 20) for N <= 18,
-// (8, 3, 26) for N <= 24, (32, 1, 34) above; FP64 (whose rows take twice the
-// registers): (16, 2, 20), (32, 1, 26), (32, 1, 34).
+template <int G, int R, bool STEP>
+cudaError_t launch_null64(hpt_system s, int64_t p, const void* ext, const void* y, void* dE, void* dN, int32_t* ok,
+                          const hpt_paths& S, const hpt_params& prm, cudaStream_t st) {
+  cudaError_t e = qr_smem_attr(null64_kernel<G, R, STEP>, lu64_smem<G>(G * R));
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = (p + lu64_paths<G>() - 1) / lu64_paths<G>();
+  if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+  int pi = prof_begin(s, STEP ? "qr_step" : "qr_directions", st);
+  null64_kernel<G, R, STEP><<<(unsigned)blocks, kLuThreads, lu64_smem<G>(s->nv), st>>>(
+      s->n, s->nv, s->proj, p, (const double2*)ext, (const double2*)y, (double2*)dE, (double2*)dN, ok, S, prm);
+  prof_end(s, pi, st);
+  return cudaGetLastError();
+}
+
+// Shapes by N = nv: FP64 as the LU solves (lu_shape); FP32 reflectors (CM >=
+// N + 2 columns in registers) (G, R, CM) = (8, 1, 10) for N <= 8, (8, 2, 18)
+// for N <= 16, (8, 3, 20) for N <= 18, (8, 3, 26) for N <= 24, (32, 1, 34)
+// above.
 template <bool STEP>
 cudaError_t launch_qr_any(hpt_system s, int64_t p, const void* ext, const void* y, void* dE, void* dN, int32_t* ok,
                           const hpt_paths& S, const hpt_params& prm, cudaStream_t st) {
   if (p <= 0) return cudaSuccess;
   const int N = s->nv;
   if (s->prec == HPT_FP64) {
-    if (N <= 8) return launch_qr_shape<double, 8, 1, 10, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
-    if (N <= 16) return launch_qr_shape<double, 8, 2, 18, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
-    if (N <= 18) return launch_qr_shape<double, 16, 2, 20, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
-    if (N <= 24) return launch_qr_shape<double, 32, 1, 26, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
-    return launch_qr_shape<double, 32, 1, 34, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
+    const int sh = lu_shape(N, p);
+    return sh == 0 ? launch_null64<8, 1, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
+         : sh == 1 ? launch_null64<8, 2, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
+         : sh == 2 ? launch_null64<16, 2, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
+                   : launch_null64<32, 1, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
   }
   if (N <= 8) return launch_qr_shape<float, 8, 1, 10, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
   if (N <= 16) return launch_qr_shape<float, 8, 2, 18, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);

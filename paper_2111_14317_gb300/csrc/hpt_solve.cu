@@ -1037,7 +1037,7 @@ step_fp64_kernel(int n, int64_t p, const double2* __restrict__ ext, hpt_paths S,
   {
     const int i = threadIdx.x % P;
     const int64_t qi = q0 + i;
-    lu64_stage<G>(n, n, ext, qi, qi < p && S.status[qi] == HPT_PATH_ACTIVE, mats + i * stride, false);
+    lu64_stage<G>(n, n, n, ext, qi, qi < p && S.status[qi] == HPT_PATH_ACTIVE, mats + i * stride, false);
   }
   const int64_t path = q0 + g;
   const int32_t status = path < p ? S.status[path] : -1;
@@ -1081,7 +1081,7 @@ newton_kernel(int n0, int64_t p, const double2* __restrict__ ext, double2* __res
   {
     const int i = threadIdx.x % P;
     const int64_t qi = q0 + i, pi = qi < end ? (MAP ? pm.list[qi] : qi) : -1;
-    lu64_stage<G>(n, MAP ? pm.nmax : n, ext, qi, pi >= 0 && done[pi] == 0, mats + i * stride, false);
+    lu64_stage<G>(n, n, MAP ? pm.nmax : n, ext, qi, pi >= 0 && done[pi] == 0, mats + i * stride, false);
   }
   const int64_t q = q0 + g;
   const int64_t path = q < end ? (MAP ? pm.list[q] : q) : -1;
@@ -1148,7 +1148,7 @@ adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, c
   double2* mats = (double2*)smem;
   {
     const int i = threadIdx.x % P;
-    lu64_stage<G>(n, n, ext, q0 + i, q0 + i < p, mats + i * stride, true);
+    lu64_stage<G>(n, n, n, ext, q0 + i, q0 + i < p, mats + i * stride, true);
   }
   const int64_t path = q0 + g;
   const bool valid = path < p;
@@ -1396,18 +1396,6 @@ cudaError_t launch_redo_shape(const StepArgs& a, cudaStream_t st) {
   const unsigned nb = blocks_for(std::min<int64_t>(a.p, 8192) * G, kSolveThreads);
   redo_fp64_kernel<G, R><<<nb, kSolveThreads, smem, st>>>(a.n, a.ext, a.st, a.prm, a.redo_count, a.redo_list, pm);
   return cudaGetLastError();
-}
-
-// The FP64 solves: (G, R) = (8, 1) for n <= 8, (8, 2) for n <= 16, (16, 2) for
-// n <= 32 where the paths fill the chip; 32 lanes a path where fewer than
-// kLuWarps warps would be in flight: a path's chain is then shorter (the
-// lanes that a step's entries do not fill cost nothing on an idle pipe).
-// Every shape gives the same bits.
-constexpr int64_t kLuWarps = 152 * 4 * 2;
-inline int lu_shape(int n, int64_t p) {
-  const int G = n <= 16 ? 8 : 16;
-  if (p * G < 32 * kLuWarps) return 3;
-  return n <= 8 ? 0 : (n <= 16 ? 1 : 2);
 }
 
 template <int G, int R>
