@@ -155,6 +155,57 @@ eval_fp64_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const doub
   }
 }
 
+// One monomial of the fixed-point evaluation.  op. 2 of Algorithm 2: W = log c
+// + [z, tau] . A[:, i] ..
+__device__ __forceinline__ void fx_begin(const FxMono& m, const fx::Wide& tw, float tf, int64_t& W, uint64_t& th,
+                                         float& wf) {
+  W = m.lc;
+  th = m.turn;
+  wf = fmaf(m.ef, tf, m.lcf);
+  if (m.e) W += fx::times((int64_t)m.e, tw);
+}
+__device__ __forceinline__ void fx_add(const FxEnt& e, const ulonglong2* zl, const float* ll, int64_t& W,
+                                       uint64_t& th, float& wf) {
+  const ulonglong2 z = zl[e.j * 32];
+  W += (int64_t)e.a * (int64_t)z.x;
+  th += (uint64_t)((int64_t)e.a * (int64_t)z.y);
+  wf = fmaf((float)e.a, ll[e.j * 32], wf);
+}
+// .. and its value times (a, e/D, 1), accumulated over the equation's
+// monomials.
+__device__ __forceinline__ void fx_accumulate(const FxMono& m, const FxEnt* __restrict__ en, double er, double ei,
+                                              double2* acc, double2& accT, double2& accH) {
+  accH.x += er;
+  accH.y += ei;
+  if (m.e) {
+    accT.x = fma(m.eD, er, accT.x);
+    accT.y = fma(m.eD, ei, accT.y);
+  }
+  int t = 0;
+  for (; t + 4 <= m.nnz; t += 4) {
+    double2 v[4];
+    FxEnt x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = en[t + u];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = acc[x[u].j * 32];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u].x = fma(x[u].ad, er, v[u].x);
+      v[u].y = fma(x[u].ad, ei, v[u].y);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[x[u].j * 32] = v[u];   // the entries of a monomial are distinct
+  }
+  for (; t < m.nnz; ++t) {
+    const FxEnt x = en[t];
+    double2 v = acc[x.j * 32];
+    v.x = fma(x.ad, er, v.x);
+    v.y = fma(x.ad, ei, v.y);
+    acc[x.j * 32] = v;
+  }
+}
+
 // The fixed-point evaluation.  A block of four warps owns 32 points, one per
 // lane; warp w takes the equations 4 g + w of its group g = blockIdx.y (groups
 // share a tile's points, so that few tiles still fill the chip).
@@ -256,54 +307,37 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
     for (int u = 0; u < nv; ++u) acc[u * 32] = make_double2(0.0, 0.0);
     double2 accT = make_double2(0.0, 0.0), accH = make_double2(0.0, 0.0);
     const int i0 = S.off[k], i1 = i0 + S.msz[k];
-    for (int i = i0; i < i1; ++i) {
-      // op. 2 of Algorithm 2, one monomial: W = log c + [z, tau] . A[:, i]
-      const FxMono m = S.mono[i];
-      const FxEnt* __restrict__ en = S.ent + m.ent;
-      int64_t W = m.lc;
-      uint64_t th = m.turn;
-      float wf = fmaf(m.ef, tf, m.lcf);
-      if (m.e) W += fx::times((int64_t)m.e, tw);
-#pragma unroll 4
-      for (int t = 0; t < m.nnz; ++t) {
-        const int a = en[t].a, j = en[t].j;
-        const ulonglong2 z = zl[j * 32];
-        W += (int64_t)a * (int64_t)z.x;
-        th += (uint64_t)((int64_t)a * (int64_t)z.y);
-        wf = fmaf((float)a, ll[j * 32], wf);
-      }
-      double er, ei;
-      fx::exp_of(W, th, wf, exp1, exp2, cs1, cs2, er, ei);
-      // ... times (a, e/D, 1), accumulated over the equation's monomials
-      accH.x += er;
-      accH.y += ei;
-      if (m.e) {
-        accT.x = fma(m.eD, er, accT.x);
-        accT.y = fma(m.eD, ei, accT.y);
-      }
+    // two monomials at a time: their integer chains interleave (1.075 -> 1.048 ms
+    // at the size above, 43 -> 39 us at n = 24, 1,000 points)
+    for (int i = i0; i < i1; i += 2) {
+      const int two = i + 1 < i1;   // the last one of an odd support stands in for its partner
+      const FxMono m0 = S.mono[i], m1 = S.mono[i + two];
+      const FxEnt* __restrict__ e0 = S.ent + m0.ent;
+      const FxEnt* __restrict__ e1 = S.ent + m1.ent;
+      int64_t W0, W1;
+      uint64_t th0, th1;
+      float wf0, wf1;
+      fx_begin(m0, tw, tf, W0, th0, wf0);
+      fx_begin(m1, tw, tf, W1, th1, wf1);
+      const int both = min(m0.nnz, m1.nnz);
       int t = 0;
-      for (; t + 4 <= m.nnz; t += 4) {
-        double2 v[4];
-        FxEnt x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = en[t + u];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = acc[x[u].j * 32];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          v[u].x = fma(x[u].ad, er, v[u].x);
-          v[u].y = fma(x[u].ad, ei, v[u].y);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[x[u].j * 32] = v[u];   // the entries of a monomial are distinct
+#pragma unroll 4
+      for (; t < both; ++t) {
+        fx_add(e0[t], zl, ll, W0, th0, wf0);
+        fx_add(e1[t], zl, ll, W1, th1, wf1);
       }
-      for (; t < m.nnz; ++t) {
-        const FxEnt x = en[t];
-        double2 v = acc[x.j * 32];
-        v.x = fma(x.ad, er, v.x);
-        v.y = fma(x.ad, ei, v.y);
-        acc[x.j * 32] = v;
+      for (int u = t; u < m0.nnz; ++u) fx_add(e0[u], zl, ll, W0, th0, wf0);
+      for (int u = t; u < m1.nnz; ++u) fx_add(e1[u], zl, ll, W1, th1, wf1);
+      double er0, ei0, er1, ei1;
+      if (fx::exp_in_range(wf0) && fx::exp_in_range(wf1)) {
+        fx::exp_in(W0, th0, wf0, exp1, exp2, cs1, cs2, er0, ei0);
+        fx::exp_in(W1, th1, wf1, exp1, exp2, cs1, cs2, er1, ei1);
+      } else {
+        fx::exp_of(W0, th0, wf0, exp1, exp2, cs1, cs2, er0, ei0);
+        fx::exp_of(W1, th1, wf1, exp1, exp2, cs1, cs2, er1, ei1);
       }
+      fx_accumulate(m0, e0, er0, ei0, acc, accT, accH);
+      if (two) fx_accumulate(m1, e1, er1, ei1, acc, accT, accH);
     }
     if (path < 0) continue;
     // a row whose sum is not finite (a point without a logarithm, a monomial

@@ -24,6 +24,7 @@
 // Qn below means a fixed-point number with n fraction bits.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -357,31 +358,50 @@ HPT_FX int64_t exp2_frac(int64_t W, const int64_t* exp1, const int64_t* exp2) {
   const int64_t h = g + mul62(g, s);
   return e + (mul62(e, h) >> 12);
 }
-// v 2^(k - 62) rounded to double (k within the exponent range of a double).
+// v 2^(k - 62) rounded to double, for results in the normal range (or v = 0).
 HPT_FX double to_double(int64_t v, int k) {
   const uint64_t neg = (uint64_t)(v >> 63);
   uint64_t m = ((uint64_t)v ^ neg) - neg;
-  if (m == 0) return 0.0;
-  const int lz = clz64(m);
+  const int lz = clz64(m | 1);
   m <<= lz;
-  int e = k + 1 - lz + 1023;   // biased exponent of the leading bit
-  if (e < 1) {                 // subnormal result
-    if (e < -60) return of_bits(neg << 63);
-    m >>= 1 - e;
-    return of_bits((((m >> 10) + 1) >> 1) | (neg << 63));
-  }
-  return of_bits((((uint64_t)(e - 1) << 52) + (((m >> 10) + 1) >> 1)) | (neg << 63));
+  const uint64_t b = ((uint64_t)(k + 1023 - lz) << 52) + (((m >> 10) + 1) >> 1);   // the leading bit adds 1 to the exponent
+  return of_bits(v == 0 ? 0 : b | (neg << 63));
+}
+// The same near and past the ends of the range: subnormal results, zero,
+// infinity.
+HPT_FX double to_double_any(int64_t v, int k) {
+  if (k > 900) return to_double(v, k - 600) * 4.149515568880993e180;                         // 2^600
+  if (k < -900) return k < -1200 ? 0.0 : to_double(v, k + 600) * 2.409919865102884e-181;     // 2^-600
+  return to_double(v, k);
 }
 
 // The value of an exponent sum: 2^W (cos, sin)(2 pi turn), from the sum W
-// modulo 16 (Q60), the phase and W in FP32 (within 7 of W).  Past the range
-// of a double: 0, or NaN (over).
-HPT_FX void exp_of(int64_t W, uint64_t turn, float wf, const int64_t* exp1, const int64_t* exp2,
-                   const int64_t (*cs1)[2], const int64_t (*cs2)[2], double& er, double& ei) {
+// modulo 16 (Q60), the phase and W in FP32 (within 7 of W).  exp_in: |wf| <=
+// 900, no branches, so that a caller can interleave several; exp_of: every
+// wf; past the range of a double 0, or NaN (over).
+HPT_FX int exponent_of(int64_t W, float wf) {
   const int k4 = (int)(W >> 60);   // integer part modulo 16, in [-8, 8)
+#ifdef __CUDA_ARCH__
+  return k4 + 16 * __float2int_rn((wf - (float)k4) * 0.0625f);
+#else
+  return k4 + 16 * (int)lrintf((wf - (float)k4) * 0.0625f);
+#endif
+}
+HPT_FX void exp_in(int64_t W, uint64_t turn, float wf, const int64_t* exp1, const int64_t* exp2,
+                   const int64_t (*cs1)[2], const int64_t (*cs2)[2], double& er, double& ei) {
   int64_t c, s;
   cossin(turn, cs1, cs2, c, s);
   const int64_t m = exp2_frac(W, exp1, exp2);
+  const int k = exponent_of(W, wf);
+  er = to_double(mul62(m, c), k);
+  ei = to_double(mul62(m, s), k);
+}
+HPT_FX bool exp_in_range(float wf) { return wf <= 900.f && wf >= -900.f; }
+#ifdef __CUDACC__
+__host__ __device__ __noinline__
+#endif
+static void exp_of(int64_t W, uint64_t turn, float wf, const int64_t* exp1, const int64_t* exp2,
+                    const int64_t (*cs1)[2], const int64_t (*cs2)[2], double& er, double& ei) {
   if (!(wf < 1030.f)) {   // over the range, or a NaN in the sum
     er = ei = of_bits((uint64_t)0x7ff8 << 48);
     return;
@@ -390,15 +410,12 @@ HPT_FX void exp_of(int64_t W, uint64_t turn, float wf, const int64_t* exp1, cons
     er = ei = 0.0;
     return;
   }
-  const float q = (wf - (float)k4) * 0.0625f;
-  const int k = k4 + 16 * (int)(q >= 0.f ? q + 0.5f : q - 0.5f);
-  if (k > 1020) {   // near the range's end: scaled so that rounding overflows to infinity as it should
-    er = to_double(mul62(m, c), k - 16) * 65536.0;
-    ei = to_double(mul62(m, s), k - 16) * 65536.0;
-    return;
-  }
-  er = to_double(mul62(m, c), k);
-  ei = to_double(mul62(m, s), k);
+  int64_t c, s;
+  cossin(turn, cs1, cs2, c, s);
+  const int64_t m = exp2_frac(W, exp1, exp2);
+  const int k = exponent_of(W, wf);
+  er = to_double_any(mul62(m, c), k);
+  ei = to_double_any(mul62(m, s), k);
 }
 
 }  // namespace fx

@@ -1195,7 +1195,8 @@ adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, c
         th += (uint64_t)((int64_t)a * (int64_t)z.y);
         wf = fmaf((float)a, lfs[g][j], wf);
       }
-      fx::exp_of(W, th, wf, T.exp1, T.exp2, T.cs1, T.cs2, mr, mi);
+      if (fx::exp_in_range(wf)) fx::exp_in(W, th, wf, T.exp1, T.exp2, T.cs1, T.cs2, mr, mi);
+      else fx::exp_of(W, th, wf, T.exp1, T.exp2, T.cs1, T.cs2, mr, mi);
     } else {
       const double* ai = sys.ahat + (size_t)i * (n + 1);
       double wr = 0.0, wi = 0.0;
