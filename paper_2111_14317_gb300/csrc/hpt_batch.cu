@@ -64,7 +64,9 @@ struct hpt_batch_s {
   int32_t* h_ctl = nullptr;       // pinned copy of the control words
 
   cudaStream_t own = nullptr;
+  cudaStream_t side[hpt::kBuckets] = {};   // branches of a captured round: the buckets' solves
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join[hpt::kBuckets] = {};
 
   // captured round and the key it was captured for
   cudaGraphExec_t exec = nullptr;
@@ -333,14 +335,32 @@ cudaError_t enqueue_round(hpt_batch_s* b, const Problem& q, const hpt_params& pr
     a.err = b->d_err;
     a.redo_count = (int32_t*)(d + q.o_rc);
     a.redo_list = (int64_t*)(d + q.o_rl);
+    // the buckets' solves touch different paths: branches of the graph, so
+    // that a step waits for the longest of them instead of their sum
+    bool first = true;
     for (int bk = 0; bk < kBuckets && e == cudaSuccess; ++bk) {
       if (!q.cap_bucket[bk]) continue;
       a.p = q.cap_bucket[bk];
       a.map = pm;
       a.map.pos_begin = ctl + 1 + bk;
       a.map.npos = ctl + 1 + kBuckets + bk;
-      e = launch_solve_fp32_shape(fp32_shape(b, bk), a, st);
+      cudaStream_t sb = st;
+      if (first) {
+        e = cudaEventRecord(b->ev_fork, st);
+      } else {
+        sb = b->side[bk];
+        e = cudaStreamWaitEvent(sb, b->ev_fork, 0);
+      }
+      if (e == cudaSuccess) e = launch_solve_fp32_shape(fp32_shape(b, bk), a, sb);
       ++nk;
+      if (!first && e == cudaSuccess) e = cudaEventRecord(b->ev_join[bk], sb);
+      first = false;
+    }
+    first = true;
+    for (int bk = 0; bk < kBuckets && e == cudaSuccess; ++bk) {
+      if (!q.cap_bucket[bk]) continue;
+      if (!first) e = cudaStreamWaitEvent(st, b->ev_join[bk], 0);
+      first = false;
     }
     if (e != cudaSuccess) break;
     a.p = q.cap;
@@ -602,6 +622,12 @@ hpt_status hpt_batch_create(int32_t nsys, const hpt_system* systems, hpt_batch* 
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+  for (int k = 0; k < kBuckets && e == cudaSuccess; ++k) {
+    if (b->span.first[k] < 0) continue;
+    e = cudaStreamCreateWithFlags(&b->side[k], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming);
+  }
   if (e != cudaSuccess) {
     hpt_status rc = cuda_fail(e, "batch create");
     hpt_batch_destroy(b);
@@ -627,6 +653,11 @@ hpt_status hpt_batch_destroy(hpt_batch b) {
   cudaFree(b->d_state);
   if (b->h_ctl) cudaFreeHost(b->h_ctl);
   if (b->own) cudaStreamDestroy(b->own);
+  for (int k = 0; k < kBuckets; ++k) {
+    if (b->side[k]) cudaStreamDestroy(b->side[k]);
+    if (b->ev_join[k]) cudaEventDestroy(b->ev_join[k]);
+  }
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_in) cudaEventDestroy(b->ev_in);
   if (b->ev_out) cudaEventDestroy(b->ev_out);
   cudaSetDevice(prev);

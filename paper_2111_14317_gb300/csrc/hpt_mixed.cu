@@ -90,7 +90,11 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
   const int ntiles = pm.npos ? (*pm.npos + 127) / 128 : P.ntiles;
   // A CTA's work items are (tile, range of equations) pairs; the evaluation
   // of one (tile, equation) is the same whichever CTA does it.  Many
-  // systems: whole tiles, strided over the grid.  One system: the sequence
+  // systems: whole tiles, strided over the grid, or, when the tiles left are
+  // at most half the CTAs, `parts` CTAs per tile, each a contiguous part of
+  // its equations (a tile's equations are a serial chain of a few
+  // microseconds each: the tracks of 4,096 paths of 16 systems, n up to 24, with
+  // 32 of 152 SMs working took 63 ms and take 29.6, the concurrent solves included).  One system: the sequence
   // of (tile, equation) units, tile-major, is cut into gridDim.x contiguous
   // ranges of equal length (to within one unit), so every CTA does the same
   // work whether the tiles outnumber the CTAs or not; a range that crosses
@@ -99,24 +103,35 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
   const int64_t u0 = (int64_t)blockIdx.x * units / (int64_t)gridDim.x;
   const int64_t u1 = ((int64_t)blockIdx.x + 1) * units / (int64_t)gridDim.x;
   const int t0 = MAP ? 0 : (int)(u0 / P.sys.ne);
-  const int my_tiles = MAP ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
+  const int parts = MAP && ntiles > 0 ? max(1, (int)gridDim.x / ntiles) : 1;
+  const int my_tiles = MAP ? (parts > 1 ? ((int)blockIdx.x < ntiles * parts ? 1 : 0)
+                                        : (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x)
                            : (u1 > u0 ? (int)((u1 - 1) / P.sys.ne) - t0 + 1 : 0);
   if (my_tiles <= 0) return;
   const bool lookahead = P.nbuf == 2 && P.wbuf == 2;
   const int nmax = pm.nmax ? pm.nmax : P.sys.n;
-  auto tile_of = [&](int it) { return MAP ? (int)blockIdx.x + it * (int)gridDim.x : t0 + it; };
+  auto tile_of = [&](int it) {
+    return MAP ? (parts > 1 ? (int)blockIdx.x / parts : (int)blockIdx.x + it * (int)gridDim.x) : t0 + it;
+  };
   auto sys_of = [&](int tile) { return pm.tile_sys ? pm.tile_sys[tile] : 0; };
   // equations [kb, ke) of work item it (ln: the tile's equation count)
   auto krange = [&](int it, int ln, int& kb, int& ke) {
     if (MAP) {
-      kb = 0;
-      ke = ln;
+      const int part = parts > 1 ? (int)blockIdx.x % parts : 0;
+      kb = ln * part / parts;
+      ke = ln * (part + 1) / parts;
       return;
     }
     const int64_t base = (int64_t)tile_of(it) * ln;
     kb = (int)(u0 > base ? u0 - base : 0);
     ke = (int)(u1 - base < (int64_t)ln ? u1 - base : (int64_t)ln);
   };
+
+  if (MAP) {   // more parts than equations: some are empty
+    int kb, ke;
+    krange(0, pm.sys_tab[sys_of(tile_of(0))].ne, kb, ke);
+    if (kb >= ke) return;
+  }
 
   if (tid == 0) {
     // 2, 3 (W full) and 4 (J full): warps 0 and 1 commit
@@ -505,8 +520,8 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
     const int64_t units = ntiles * sys.ne;
     const int64_t per = (units + slots - 1) / slots;
     grid = per > 0 ? (units + per - 1) / per : 0;
-  } else if (grid > ntiles) {
-    grid = ntiles;
+  } else if (grid > ntiles * maxs.n) {
+    grid = ntiles * maxs.n;   // at most a CTA per (tile, equation)
   }
   if (grid < 1) return cudaSuccess;
   int pi = prof_begin(prof, "eval_mixed_tc", st);
