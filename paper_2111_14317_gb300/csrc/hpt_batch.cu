@@ -12,7 +12,7 @@
 // evaluation kernel's round-robin tile walk meets the large tiles first.
 //
 // A round is K x (evaluation over every position; per bucket the FP32 solve
-// over its range; the FP64 re-solve list) followed by the compaction (count,
+// over its range) followed by the compaction (count,
 // scan, scatter) and a read-back of the position count.  It is captured once
 // into a CUDA graph on the batch's own stream and replayed until the count
 // is 0 or the step budget is spent.
@@ -47,7 +47,6 @@ struct hpt_batch_s {
   hpt::MixedSys maxs{};   // the largest of each operand dimension
   int tmem_cols = 0;
   int nmax = 0;
-  int redo_shape = 0;
 
   // constants on the device
   uint8_t* d_chunks = nullptr;
@@ -180,7 +179,7 @@ struct Problem {
   int64_t pmax = 0;              // largest paths[s]
   // byte offsets in d_state
   size_t o_y, o_ya, o_de, o_yp, o_dp, o_tp, o_hf, o_tau, o_dt, o_ta, o_st, o_sp, o_ac, o_rj, o_sk, o_done, o_last, o_vofs,
-      o_pb, o_np, o_tmp, o_cnt, o_tb, o_list, o_tsys, o_ctl, o_rc, o_rl, o_ext, total;
+      o_pb, o_np, o_tmp, o_cnt, o_tb, o_list, o_tsys, o_ctl, o_ext, total;
 };
 
 Problem plan(const hpt_batch_s* b, const int64_t* paths) {
@@ -230,8 +229,6 @@ Problem plan(const hpt_batch_s* b, const int64_t* paths) {
   q.o_list = take((size_t)std::max<int64_t>(q.cap, 128) * 8);
   q.o_tsys = take((size_t)std::max<int64_t>(q.cap / 128, 1) * 4);
   q.o_ctl = take(kCtlWords * 4);
-  q.o_rc = take(4);
-  q.o_rl = take((size_t)std::max<int64_t>(q.cap, 1) * 8);
   // extended Jacobian of every position: complex64 while tracking,
   // complex128 while polishing
   q.o_ext = take(ext_entries(std::max<int64_t>(q.cap, 1), b->nmax) * 16);
@@ -322,8 +319,6 @@ cudaError_t enqueue_round(hpt_batch_s* b, const Problem& q, const hpt_params& pr
   int32_t nk = 0;
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < b->tune.steps_per_round && e == cudaSuccess; ++k) {
-    e = cudaMemsetAsync(d + q.o_rc, 0, 4, st);
-    if (e != cudaSuccess) break;
     e = launch_eval_mixed_map(nullptr, b->maxs, b->tmem_cols, b->d_chunks, q.cap, S.y, S.tau, pm, d + q.o_ext,
                               b->d_err, b->tune.eval_ctas_per_sm, st);
     ++nk;
@@ -333,8 +328,6 @@ cudaError_t enqueue_round(hpt_batch_s* b, const Problem& q, const hpt_params& pr
     a.st = S;
     a.prm = prm;
     a.err = b->d_err;
-    a.redo_count = (int32_t*)(d + q.o_rc);
-    a.redo_list = (int64_t*)(d + q.o_rl);
     // the buckets' solves touch different paths: branches of the graph, so
     // that a step waits for the longest of them instead of their sum
     bool first = true;
@@ -362,11 +355,6 @@ cudaError_t enqueue_round(hpt_batch_s* b, const Problem& q, const hpt_params& pr
       if (!first) e = cudaStreamWaitEvent(st, b->ev_join[bk], 0);
       first = false;
     }
-    if (e != cudaSuccess) break;
-    a.p = q.cap;
-    a.map = pm;
-    e = launch_redo_fp64_shape(b->redo_shape, a, st);
-    ++nk;
   }
   if (e == cudaSuccess) e = enqueue_compaction(b, q, S.status, HPT_PATH_ACTIVE, st);
   nk += 3;
@@ -585,7 +573,6 @@ hpt_status hpt_batch_create(int32_t nsys, const hpt_system* systems, hpt_batch* 
     // evaluation work of one tile: n equations x (exponent + coefficient GEMM + exp)
     cost[s] = (double)h->n * (h->ml.MP * (double)h->ml.KX + 3.0 * h->ml.NJ * h->ml.KC + 8.0 * h->ml.MP);
   }
-  b->redo_shape = solve_shape_of(b->nmax);
   b->order.resize(nsys);
   std::iota(b->order.begin(), b->order.end(), 0);
   std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) {

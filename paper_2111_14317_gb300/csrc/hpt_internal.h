@@ -290,8 +290,6 @@ struct StepArgs {
   hpt_paths st;
   hpt_params prm;
   int32_t* err;
-  int32_t* redo_count = nullptr;   // mixed form: FP64 re-solve list (scratch)
-  int64_t* redo_list = nullptr;
 };
 
 // Consolidated solve + update + step control.  T = double for HPT_FP64,
@@ -299,12 +297,8 @@ struct StepArgs {
 cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st);
 // The state arrays of paths q0.. of S (nv complex entries per path of cs bytes).
 hpt_paths offset_paths(const hpt_paths& S, int64_t q0, int nv, size_t cs);
-// Many-systems pieces of the mixed step: the FP32 solve of one lane-group
-// shape (shape_of(n)) over the map's position range, appending FP64
-// re-solves to a.redo_list (the caller zeroes a.redo_count once per step),
-// and the FP64 re-solve of the whole list with a shape that covers a.map.nmax
-// (shapes: 0, 1, 2 as solve_shape_of, kShape8x3 for the FP32 solve).
-int solve_shape_of(int n);
+// Many-systems piece of the mixed step: the FP32 solve of one lane-group shape
+// (0: n <= 8, 1: n <= 16, 2: n <= 32, kShape8x3) over the map's position range.
 constexpr int kShape8x3 = 3;   // FP32 solve only: 8 lanes x 3 rows per path, n <= 24
 // FP64 Newton polish update over the position range [*pm.pos_begin,
 // *pm.npos) of a map (systems of n <= nbound; cap bounds the range's length); x is
@@ -313,7 +307,6 @@ constexpr int kShape8x3 = 3;   // FP32 solve only: 8 lanes x 3 rows per path, n 
 cudaError_t launch_newton_map(int nbound, int64_t cap, const void* ext, void* x, int32_t* done, float* last,
                               double tol, const PathMap& pm, cudaStream_t st);
 cudaError_t launch_solve_fp32_shape(int shape, const StepArgs& a, cudaStream_t st);
-cudaError_t launch_redo_fp64_shape(int shape, const StepArgs& a, cudaStream_t st);
 
 // Newton update at t = 1 for the polish: x += dN where the path is not done;
 // done[q] set once the error left is below tol (last[q]: the previous

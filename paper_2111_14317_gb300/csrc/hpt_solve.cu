@@ -65,12 +65,11 @@ struct PathRows {
 };
 
 
-// Loads the rows of [D_z H | -H_tau | -H] (adjoint = false) or of
-// [(D_z H)^H | g | 0] (adjoint = true, g from gx) for one path; returns
-// whether every entry is finite (group-uniform).
-template <typename T, typename S, int G, int R>
-__device__ __forceinline__ bool load_rows(int n, int nmax, const void* ext, int64_t q, size_t vbase, bool valid,
-                                          bool adjoint, const double2* gx, PathRows<T, G, R>& P) {
+// Loads the rows of [D_z H | -H_tau | -H] of one path; returns whether every
+// entry is finite (group-uniform).
+template <typename T, int G, int R>
+__device__ __forceinline__ bool load_rows(int n, int nmax, const void* ext, int64_t q, bool valid,
+                                          PathRows<T, G, R>& P) {
   constexpr int NC = G * R;
   const int lane = threadIdx.x & (G - 1);
   T chk = T(0);
@@ -82,23 +81,17 @@ __device__ __forceinline__ bool load_rows(int n, int nmax, const void* ext, int6
     for (int c = 0; c < NC; ++c) {
       P.a[s][c] = mk<T>(0, 0);
       if (have && c < n) {
-        cx<S> v = adjoint ? ld<S>(ext, ext_index(q, c, r, nmax)) : ld<S>(ext, ext_index(q, r, c, nmax));
-        P.a[s][c] = adjoint ? mk<T>((T)v.x, -(T)v.y) : mk<T>((T)v.x, (T)v.y);
+        P.a[s][c] = ld<T>(ext, ext_index(q, r, c, nmax));
         chk += t_abs(P.a[s][c].x) + t_abs(P.a[s][c].y);
       }
     }
     P.bE[s] = mk<T>(0, 0);
     P.bN[s] = mk<T>(0, 0);
     if (have) {
-      if (adjoint) {
-        const double2 g = gx[vbase + r];
-        P.bE[s] = mk<T>((T)g.x, (T)g.y);
-      } else {
-        const cx<S> ht = ld<S>(ext, ext_index(q, r, n, nmax));
-        const cx<S> h = ld<S>(ext, ext_index(q, r, n + 1, nmax));
-        P.bE[s] = mk<T>(-(T)ht.x, -(T)ht.y);
-        P.bN[s] = mk<T>(-(T)h.x, -(T)h.y);
-      }
+      const cx<T> ht = ld<T>(ext, ext_index(q, r, n, nmax));
+      const cx<T> h = ld<T>(ext, ext_index(q, r, n + 1, nmax));
+      P.bE[s] = mk<T>(-ht.x, -ht.y);
+      P.bN[s] = mk<T>(-h.x, -h.y);
       chk += t_abs(P.bE[s].x) + t_abs(P.bE[s].y) + t_abs(P.bN[s].x) + t_abs(P.bN[s].y);
     }
   }
@@ -583,45 +576,82 @@ __device__ __forceinline__ size_t pm_vbase(const PathMap& m, int64_t path, int n
 __device__ __forceinline__ int64_t pm_count(const PathMap& m, int64_t p) { return m.npos ? (int64_t)*m.npos : p; }
 __device__ __forceinline__ int64_t pm_begin(const PathMap& m) { return m.pos_begin ? (int64_t)*m.pos_begin : 0; }
 
-// One Euler-Newton step per ACTIVE path: consolidated solve, then the step
-// control.  T is the state and solve precision.  FP32 solves whose pivot
-// ratio (after equilibration) exceeds prm.cond_max are not applied here: the
-// position goes to redo_list and is solved again in FP64 by redo_fp64_kernel.
-// One system: G threads per path, a grid that covers every path once.  The
-// FP32 8-lane two-row form is register-capped for five resident blocks per
-// SM (shared memory allows five): more warps to cover each warp's dependent
-// chain of loads, shuffles and shared-memory round trips.
-template <typename T, int G, int R>
-__global__ void __launch_bounds__(kSolveThreads, (sizeof(T) == 4 && G == 8 && R == 2) ? 5 : 1)
-solve_update_kernel(int n, int64_t p, const void* __restrict__ ext, hpt_paths S, hpt_params prm,
-                    int32_t* __restrict__ redo_count, int64_t* __restrict__ redo_list) {
+// FP64 re-solve of the paths that a warp's FP32 solves flagged (pivot ratio
+// above prm.cond_max): same FP32 Jacobian, FP64 factorisation, then the step
+// control in the FP32 state, one path after another with all 32 lanes, in the
+// warp's own shared memory (W: lu64_entries + lu64_col_entries of n).  Flagged
+// paths are rare; a launch of their own, with its list and counter to clear,
+// cost every step 6 us whether there was one or not (250 paths, n = 14: 28.7
+// -> 22.6 us a step; 65,536 paths, n = 16: 212 -> 206 us, and with every path
+// flagged 4.2 -> 2.4 ms).  Call with the warp
+// converged; flag and the path's data are group-uniform.
+__device__ __noinline__ void resolve_flagged(int G, bool flag, int n, int nmax, int64_t q, int64_t path, size_t vbase,
+                                             const float2* __restrict__ ext, const hpt_paths& S,
+                                             const hpt_params& prm, double2* W) {
+  const int lane = threadIdx.x & 31;
+  unsigned m = __ballot_sync(0xffffffffu, flag && (lane & (G - 1)) == 0);
+  while (m) {
+    const int src = __ffs(m) - 1;
+    m &= m - 1;
+    const int64_t qs = __shfl_sync(0xffffffffu, q, src), ps = __shfl_sync(0xffffffffu, path, src);
+    const size_t vs = __shfl_sync(0xffffffffu, (unsigned long long)vbase, src);
+    __syncwarp();   // the warp's shared memory is free
+    const int np2 = n + 2;
+    for (int e = lane; e < n * np2; e += 32) {
+      const int k = e / np2, u = e - k * np2;
+      const float2 v = ext[ext_index(qs, k, u, nmax)];
+      W[e] = make_double2((double)v.x, (double)v.y);
+    }
+    __syncwarp();
+    int* colx = (int*)(W + lu64_entries(n));
+    const bool ok = lu64_solve<32>(n, W, colx, -1);
+    cx<float> fE[1], fN[1];
+    fE[0] = fN[0] = mk<float>(0.f, 0.f);
+    if (lane < n) {
+      const cx<double> e = lu64_x(n, W, colx, lane, 0), f = lu64_x(n, W, colx, lane, 1);
+      fE[0] = mk<float>((float)e.x, (float)e.y);
+      fN[0] = mk<float>((float)f.x, (float)f.y);
+    }
+    update_path<float, 32, 1>(n, ps, vs, HPT_PATH_ACTIVE, ok, fE, fN, S, prm);
+    __syncwarp();
+  }
+}
+// Whether the warp has a flagged path at all (the usual answer is no).
+__device__ __forceinline__ bool any_flagged(bool flag) { return __any_sync(0xffffffffu, flag); }
+// Shared memory of one warp of a solve kernel: its groups' regions, or one
+// path's FP64 matrix, whichever is larger.
+inline int warp_smem(int groups_bytes, int n) {
+  return std::max(groups_bytes, (lu64_entries(n) + lu64_col_entries(n)) * 16);
+}
+
+// One FP32 Euler-Newton step per ACTIVE path: consolidated solve, then the
+// step control.  Solves whose pivot ratio (after equilibration) exceeds
+// prm.cond_max are not applied but solved again in FP64 (resolve_flagged).
+// One system, n > 16: a warp per path, a grid that covers every path once;
+// ws: bytes of shared memory per warp.
+__global__ void __launch_bounds__(kSolveThreads)
+solve_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
+                    const __grid_constant__ hpt_params prm, int ws) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & (G - 1);
-  const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int32_t status = path < p ? S.status[path] : -1;
   const bool valid = status == HPT_PATH_ACTIVE;
-  unsigned char* sm = smem + (threadIdx.x / G) * GroupSmem<T, G * R>::bytes;
-  if (G == 32) {   // block-uniform: stage the block's four paths
-    const int64_t q0 = (int64_t)blockIdx.x * (kSolveThreads / 32);
-    const int64_t qi = q0 + (threadIdx.x & 3);
-    stage_block_rows<T>(n, n, ext, q0, qi < p && S.status[qi] == HPT_PATH_ACTIVE, smem, GroupSmem<T, G * R>::bytes);
-    __syncthreads();
-  }
-  if (!__any_sync(0xffffffffu, valid)) return;   // warp-uniform exit
+  unsigned char* sm = smem + (threadIdx.x / 32) * ws;
+  const int64_t q0 = (int64_t)blockIdx.x * (kSolveThreads / 32);
+  const int64_t qi = q0 + (threadIdx.x & 3);
+  stage_block_rows<float>(n, n, ext, q0, qi < p && S.status[qi] == HPT_PATH_ACTIVE, smem, ws);
+  __syncthreads();
+  if (!valid) return;   // warp-uniform
   const size_t vbase = (size_t)path * n;
-  PathRows<T, G, R> P;
-  bool fin;
-  if constexpr (G == 32) fin = load_rows_staged<T, T>(n, sm, valid, P);
-  else fin = load_rows<T, T, G, R>(n, n, ext, path, vbase, valid, false, nullptr, P);
-  cx<T> xE[R], xN[R];
-  T cond;
-  const bool ok = group_solve<T, G, R>(n, P, xE, xN, cond, sm) && fin;
-  if (!valid) return;   // group-uniform; only group-masked shuffles below
-  if (sizeof(T) == 4 && redo_list && ok && !(cond <= (T)prm.cond_max)) {
-    if (lane == 0) redo_list[atomicAdd(redo_count, 1)] = path;
-    return;
-  }
-  update_path<T, G, R>(n, path, vbase, status, ok, xE, xN, S, prm);
+  PathRows<float, 32, 1> P;
+  const bool fin = load_rows_staged<float, float>(n, sm, valid, P);
+  cx<float> xE[1], xN[1];
+  float cond;
+  const bool ok = group_solve<float, 32, 1>(n, P, xE, xN, cond, sm) && fin;
+  if (ok && !(cond <= (float)prm.cond_max))
+    resolve_flagged(32, true, n, n, path, path, vbase, ext, S, prm, (double2*)sm);
+  else
+    update_path<float, 32, 1>(n, path, vbase, status, ok, xE, xN, S, prm);
 }
 
 // FP32 step of one system with n <= G R by Gauss-Jordan elimination.  A
@@ -669,16 +699,16 @@ __device__ __forceinline__ float cmag2(uint64_t v) {
 
 // One path (position q of the scratch, laid out for nmax variables) for
 // every lane of its group; call with the whole warp converged.  Returns with
-// the state updated, or the position queued for the FP64 re-solve.
+// the state updated, or true (group-uniform): to be solved again in FP64.
+// smem is the group's.
 template <int G, int R>
-__device__ __forceinline__ void gj_path(int n, int nmax, int64_t q, int64_t path, size_t vbase, int32_t status,
+__device__ __forceinline__ bool gj_path(int n, int nmax, int64_t q, int64_t path, size_t vbase, int32_t status,
                                         const float2* __restrict__ ext, const hpt_paths& S, const hpt_params& prm,
-                                        int32_t* __restrict__ redo_count, int64_t* __restrict__ redo_list,
                                         unsigned char* smem) {
   constexpr int NC = G * R;
   const int lane = threadIdx.x & (G - 1);
   const bool valid = status == HPT_PATH_ACTIVE;
-  GjSmem<NC>& sh = *(GjSmem<NC>*)(smem + (threadIdx.x / G) * GjLayout<G, NC>::bytes);
+  GjSmem<NC>& sh = *(GjSmem<NC>*)smem;
   const unsigned gmask = group_mask<G>();
 
   // rows lane + G s and their right-hand sides
@@ -871,23 +901,32 @@ __device__ __forceinline__ void gj_path(int n, int nmax, int64_t q, int64_t path
   const float cond = pmin > 0.f ? sqrtf(pmax / pmin) : INFINITY;
   ok = ok && fin;
   __syncwarp();   // the group's shared memory is reused by its next path
-  if (!valid) return;   // group-uniform; only group-masked shuffles below
-  if (redo_list && ok && !(cond <= (float)prm.cond_max)) {
-    if (lane == 0) redo_list[atomicAdd(redo_count, 1)] = q;
-    return;
-  }
+  if (!valid) return false;   // group-uniform; only group-masked shuffles below
+  if (ok && !(cond <= (float)prm.cond_max)) return true;
   update_path<float, G, R>(n, path, vbase, status, ok, wE, wN, S, prm);
+  return false;
+}
+// Bytes of a warp: its groups' regions; they also hold one path's FP64 matrix.
+template <int G, int R>
+__host__ __device__ constexpr int gj_warp_bytes() {
+  static_assert((32 / G) * GjLayout<G, G * R>::bytes >= (G * R * (G * R + 2) + 1 + (G * R + 3) / 4) * 16,
+                "a warp's regions hold one path's FP64 matrix");
+  return (32 / G) * GjLayout<G, G * R>::bytes;
 }
 
 template <int G, int R>
 __global__ void __launch_bounds__(kSolveThreads, R == 1 ? 6 : 4)
-gj_update_kernel(int n, int64_t p, const float2* __restrict__ ext, hpt_paths S, hpt_params prm,
-                 int32_t* __restrict__ redo_count, int64_t* __restrict__ redo_list) {
+gj_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
+                 const __grid_constant__ hpt_params prm) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int32_t status = path < p ? S.status[path] : -1;
   if (!__any_sync(0xffffffffu, status == HPT_PATH_ACTIVE)) return;   // warp-uniform exit
-  gj_path<G, R>(n, n, path, path, (size_t)path * n, status, ext, S, prm, redo_count, redo_list, smem);
+  const bool again = gj_path<G, R>(n, n, path, path, (size_t)path * n, status, ext, S, prm,
+                                   smem + (threadIdx.x / G) * GjLayout<G, G * R>::bytes);
+  if (any_flagged(again))
+    resolve_flagged(G, again, n, n, path, path, (size_t)path * n, ext, S, prm,
+                    (double2*)(smem + (threadIdx.x / 32) * gj_warp_bytes<G, R>()));
 }
 
 // The same over a position map (many systems), persistent as
@@ -895,8 +934,8 @@ gj_update_kernel(int n, int64_t p, const float2* __restrict__ ext, hpt_paths S, 
 // 128-position tile, so n is warp-uniform.
 template <int G, int R>
 __global__ void __launch_bounds__(kSolveThreads, R == 1 ? 6 : 4)
-gj_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, hpt_paths S, hpt_params prm,
-                     int32_t* __restrict__ redo_count, int64_t* __restrict__ redo_list, PathMap pm) {
+gj_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
+                     const __grid_constant__ hpt_params prm, PathMap pm) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int per_warp = 32 / G;
   const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
@@ -910,24 +949,29 @@ gj_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, hpt_path
     const int32_t status = path >= 0 ? S.status[path] : -1;
     if (!__any_sync(0xffffffffu, status == HPT_PATH_ACTIVE)) continue;   // warp-uniform skip
     const size_t vbase = status == HPT_PATH_ACTIVE ? pm_vbase(pm, path, n) : 0;
-    gj_path<G, R>(n, pm.nmax, q, path, vbase, status, ext, S, prm, redo_count, redo_list, smem);
+    const bool again = gj_path<G, R>(n, pm.nmax, q, path, vbase, status, ext, S, prm,
+                                     smem + (threadIdx.x / G) * GjLayout<G, G * R>::bytes);
+    if (any_flagged(again))
+      resolve_flagged(G, again, n, pm.nmax, q, path, vbase, ext, S, prm,
+                      (double2*)(smem + (threadIdx.x / 32) * gj_warp_bytes<G, R>()));
   }
 }
 
 // The same over a position map (many systems).  Persistent: the warps loop
 // over the positions of [*pos_begin, *npos) (32/G consecutive positions per
 // warp, always inside one 128-position tile, so n is warp-uniform).
-template <typename T, int G, int R>
+template <int G, int R>
 __global__ void __launch_bounds__(kSolveThreads)
-solve_update_map_kernel(int n0, int64_t p, const void* __restrict__ ext, hpt_paths S, hpt_params prm,
-                        int32_t* __restrict__ redo_count, int64_t* __restrict__ redo_list, PathMap pm) {
+solve_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
+                        const __grid_constant__ hpt_params prm, PathMap pm, int ws) {
+  typedef float T;
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int per_warp = 32 / G;
-  const int lane = threadIdx.x & (G - 1);
   const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
   const int g = (threadIdx.x & 31) / G;
-  unsigned char* sm = smem + (threadIdx.x / G) * GroupSmem<T, G * R>::bytes;
+  unsigned char* wsm = smem + (threadIdx.x / 32) * ws;
+  unsigned char* sm = wsm + g * GroupSmem<T, G * R>::bytes;
   const int64_t npos = pm_count(pm, p);
   const int nmax = pm.nmax;
   // with 32-lane groups the block's four warps take consecutive positions of
@@ -943,8 +987,7 @@ solve_update_map_kernel(int n0, int64_t p, const void* __restrict__ ext, hpt_pat
       const int64_t q0 = base - (threadIdx.x >> 5);
       const int64_t pi = pm_path(pm, q0 + (threadIdx.x & 3));
       __syncthreads();   // the previous iteration's solves are done with the regions
-      stage_block_rows<T>(n, nmax, ext, q0, pi >= 0 && S.status[pi] == HPT_PATH_ACTIVE, smem,
-                          GroupSmem<T, G * R>::bytes);
+      stage_block_rows<T>(n, nmax, ext, q0, pi >= 0 && S.status[pi] == HPT_PATH_ACTIVE, smem, ws);
       __syncthreads();
     }
     if (!__any_sync(0xffffffffu, valid)) continue;   // warp-uniform skip
@@ -952,72 +995,14 @@ solve_update_map_kernel(int n0, int64_t p, const void* __restrict__ ext, hpt_pat
     PathRows<T, G, R> P;
     bool fin;
     if constexpr (G == 32) fin = load_rows_staged<T, T>(n, sm, valid, P);
-    else fin = load_rows<T, T, G, R>(n, nmax, ext, q, vbase, valid, false, nullptr, P);
+    else fin = load_rows<T, G, R>(n, nmax, ext, q, valid, P);
     cx<T> xE[R], xN[R];
     T cond;
     const bool ok = group_solve<T, G, R>(n, P, xE, xN, cond, sm) && fin;
-    if (valid) {   // group-uniform; only group-masked shuffles below
-      if (sizeof(T) == 4 && redo_list && ok && !(cond <= (T)prm.cond_max)) {
-        if (lane == 0) redo_list[atomicAdd(redo_count, 1)] = q;
-      } else {
-        update_path<T, G, R>(n, path, vbase, status, ok, xE, xN, S, prm);
-      }
-    }
+    const bool again = valid && ok && !(cond <= (T)prm.cond_max);
+    if (valid && !again) update_path<T, G, R>(n, path, vbase, status, ok, xE, xN, S, prm);   // group-uniform
     __syncwarp();
-  }
-}
-
-// FP64 re-solve of the positions listed by the FP32 kernel (same FP32
-// Jacobian, FP64 factorisation), then their step control in the FP32 state.
-// Entries of the list sit next to any other, so n may differ between the
-// groups of a warp: the warp solves with the largest n of its groups and a
-// smaller system gets identity rows for the unknowns it does not have.
-template <int G, int R>
-__global__ void __launch_bounds__(kSolveThreads)
-redo_fp64_kernel(int n0, const void* __restrict__ ext, hpt_paths S, hpt_params prm,
-                 const int32_t* __restrict__ redo_count, const int64_t* __restrict__ redo_list, PathMap pm) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int count = *redo_count;
-  constexpr int per_warp = 32 / G;
-  const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
-  const int g = (threadIdx.x & 31) / G;
-  unsigned char* sm = smem + (threadIdx.x / G) * GroupSmem<double, G * R>::bytes;
-  for (int64_t base = warp_id * per_warp; base < count; base += nwarps * per_warp) {
-    const int64_t i = base + g;
-    const bool valid = i < count;
-    const int64_t q = valid ? redo_list[i] : 0;
-    const int64_t path = valid ? pm_path(pm, q) : 0;
-    const int n = valid ? pm_n(pm, q, n0) : 0;
-    int nw = n;   // the warp's largest n: group_solve needs a warp-uniform size
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nw = max(nw, __shfl_xor_sync(0xffffffffu, nw, o));
-    const size_t vbase = valid ? pm_vbase(pm, path, n) : 0;
-    PathRows<double, G, R> P;
-    const bool fin = load_rows<double, float, G, R>(n, pm.nmax, ext, q, vbase, valid, false, nullptr, P);
-    // rows n..nw-1 become identity rows (their unknowns solve to 0)
-    const int lane = threadIdx.x & (G - 1);
-#pragma unroll
-    for (int s = 0; s < R; ++s) {
-      const int r = lane + G * s;
-      if (r >= n && r < nw) {
-#pragma unroll
-        for (int c = 0; c < G * R; ++c)
-          if (c == r) P.a[s][c] = mk<double>(1.0, 0.0);
-      }
-    }
-    cx<double> xE[R], xN[R];
-    double cond;
-    const bool ok = group_solve<double, G, R>(nw, P, xE, xN, cond, sm) && fin;
-    if (valid) {
-      cx<float> fE[R], fN[R];
-#pragma unroll
-      for (int s = 0; s < R; ++s) {
-        fE[s] = mk<float>((float)xE[s].x, (float)xE[s].y);
-        fN[s] = mk<float>((float)xN[s].x, (float)xN[s].y);
-      }
-      update_path<float, G, R>(n, path, vbase, S.status[path], ok, fE, fN, S, prm);
-    }
+    if (any_flagged(again)) resolve_flagged(G, again, n, nmax, q, path, vbase, ext, S, prm, (double2*)wsm);
     __syncwarp();
   }
 }
@@ -1347,22 +1332,16 @@ inline unsigned solve_grid(int64_t p, int G) {
   return (unsigned)std::min<int64_t>(need, (int64_t)sms * 32);
 }
 
-template <typename T, int G, int R>
-cudaError_t launch_solve_shape(const StepArgs& a, int32_t* rc, int64_t* rl, cudaStream_t st) {
-  const int smem = (kSolveThreads / G) * GroupSmem<T, G * R>::bytes;
-  if (!a.map.list) {
-    cudaError_t e = set_smem(solve_update_kernel<T, G, R>, smem);
-    if (e != cudaSuccess) return e;
-    solve_update_kernel<T, G, R><<<blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st>>>(
-        a.n, a.p, a.ext, a.st, a.prm, rc, rl);
-    return cudaGetLastError();
-  }
-  cudaError_t e = set_smem(solve_update_map_kernel<T, G, R>, smem);
-  if (e != cudaSuccess) return e;
+template <int G, int R>
+cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
-  solve_update_map_kernel<T, G, R><<<solve_grid(a.p, G), kSolveThreads, smem, st>>>(a.n, a.p, a.ext, a.st, a.prm,
-                                                                                     rc, rl, pm);
+  const int ws = warp_smem((32 / G) * GroupSmem<float, G * R>::bytes, std::min(pm.nmax, G * R));
+  const int smem = (kSolveThreads / 32) * ws;
+  cudaError_t e = set_smem(solve_update_map_kernel<G, R>, smem);
+  if (e != cudaSuccess) return e;
+  solve_update_map_kernel<G, R><<<solve_grid(a.p, G), kSolveThreads, smem, st>>>(a.n, a.p, (const float2*)a.ext, a.st,
+                                                                                  a.prm, pm, ws);
   return cudaGetLastError();
 }
 
@@ -1375,7 +1354,7 @@ cudaError_t launch_gj(const StepArgs& a, cudaStream_t st) {
     cudaError_t e = set_smem(gj_update_kernel<G, R>, smem);
     if (e != cudaSuccess) return e;
     gj_update_kernel<G, R><<<blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st>>>(
-        a.n, a.p, (const float2*)a.ext, a.st, a.prm, a.redo_count, a.redo_list);
+        a.n, a.p, (const float2*)a.ext, a.st, a.prm);
     return cudaGetLastError();
   }
   cudaError_t e = set_smem(gj_update_map_kernel<G, R>, smem);
@@ -1383,19 +1362,7 @@ cudaError_t launch_gj(const StepArgs& a, cudaStream_t st) {
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
   gj_update_map_kernel<G, R><<<solve_grid(a.p, G), kSolveThreads, smem, st>>>(
-      a.n, a.p, (const float2*)a.ext, a.st, a.prm, a.redo_count, a.redo_list, pm);
-  return cudaGetLastError();
-}
-
-template <int G, int R>
-cudaError_t launch_redo_shape(const StepArgs& a, cudaStream_t st) {
-  const int smem = (kSolveThreads / G) * GroupSmem<double, G * R>::bytes;
-  cudaError_t e = set_smem(redo_fp64_kernel<G, R>, smem);
-  if (e != cudaSuccess) return e;
-  PathMap pm = a.map;
-  if (!pm.nmax) pm.nmax = a.n;
-  const unsigned nb = blocks_for(std::min<int64_t>(a.p, 8192) * G, kSolveThreads);
-  redo_fp64_kernel<G, R><<<nb, kSolveThreads, smem, st>>>(a.n, a.ext, a.st, a.prm, a.redo_count, a.redo_list, pm);
+      a.n, a.p, (const float2*)a.ext, a.st, a.prm, pm);
   return cudaGetLastError();
 }
 
@@ -1449,7 +1416,6 @@ cudaError_t launch_adjoint_shape(hpt_system s, int64_t p, const void* ext, const
 
 cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st) {
   if (a.p <= 0) return cudaSuccess;
-  const int shape = shape_of(a.n);
   cudaError_t e;
   if (s->prec == HPT_FP64) {
     int pi = prof_begin(s, "solve_update_fp64", st);
@@ -1461,30 +1427,23 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
     prof_end(s, pi, st);
     return e;
   }
-  e = cudaMemsetAsync(a.redo_count, 0, sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
+  const int shape = shape_of(a.n);
   int pi;
-  if (!a.map.list && shape <= 1) {   // one system, n <= 16: Gauss-Jordan
+  if (shape <= 1) {   // n <= 16: Gauss-Jordan
     pi = prof_begin(s, "solve_gj_fp32", st);
     e = shape == 0 ? launch_gj<8, 1>(a, st) : launch_gj<8, 2>(a, st);
   } else {
     pi = prof_begin(s, "solve_update_fp32", st);
-    e = shape == 0 ? launch_solve_shape<float, 8, 1>(a, a.redo_count, a.redo_list, st)
-      : shape == 1 ? launch_solve_shape<float, 8, 2>(a, a.redo_count, a.redo_list, st)
-                   : launch_solve_shape<float, 32, 1>(a, a.redo_count, a.redo_list, st);
+    const int ws = warp_smem(GroupSmem<float, 32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
+    e = set_smem(solve_update_kernel, smem);
+    if (e != cudaSuccess) return e;
+    solve_update_kernel<<<blocks_for(a.p, kSolveThreads / 32), kSolveThreads, smem, st>>>(
+        a.n, a.p, (const float2*)a.ext, a.st, a.prm, ws);
+    e = cudaGetLastError();
   }
-  prof_end(s, pi, st);
-  if (e != cudaSuccess) return e;
-  // FP64 re-solves: a fixed grid that loops over the device-side list
-  pi = prof_begin(s, "redo_fp64", st);
-  e = shape == 0 ? launch_redo_shape<8, 1>(a, st)
-    : shape == 1 ? launch_redo_shape<8, 2>(a, st)
-                 : launch_redo_shape<32, 1>(a, st);
   prof_end(s, pi, st);
   return e;
 }
-
-int solve_shape_of(int n) { return shape_of(n); }
 
 cudaError_t launch_newton_map(int nbound, int64_t cap, const void* ext, void* x, int32_t* done, float* last,
                               double tol, const PathMap& pm, cudaStream_t st) {
@@ -1497,15 +1456,8 @@ cudaError_t launch_solve_fp32_shape(int shape, const StepArgs& a, cudaStream_t s
   if (a.p <= 0) return cudaSuccess;
   return shape == 0 ? launch_gj<8, 1>(a, st)
        : shape == 1 ? launch_gj<8, 2>(a, st)
-       : shape == kShape8x3 ? launch_solve_shape<float, 8, 3>(a, a.redo_count, a.redo_list, st)
-                    : launch_solve_shape<float, 32, 1>(a, a.redo_count, a.redo_list, st);
-}
-
-cudaError_t launch_redo_fp64_shape(int shape, const StepArgs& a, cudaStream_t st) {
-  if (a.p <= 0) return cudaSuccess;
-  return shape == 0 ? launch_redo_shape<8, 1>(a, st)
-       : shape == 1 ? launch_redo_shape<8, 2>(a, st)
-                    : launch_redo_shape<32, 1>(a, st);
+       : shape == kShape8x3 ? launch_solve_map<8, 3>(a, st)
+                            : launch_solve_map<32, 1>(a, st);
 }
 
 cudaError_t launch_newton_update(hpt_system s, int64_t p, const void* ext, void* x, int32_t* done,

@@ -11,8 +11,7 @@
 // exits.  Host code only holds a stand-in for its name, so the device address
 // is fetched once per device with cudaGetSymbolAddress (with that device
 // current) and cached.  All calls on a device share the array and it keeps
-// the last call's contents; the only value that must start at zero (the FP64
-// re-solve counter) is cleared by every solve launch.
+// the last call's contents; nothing in it has to start at a value.
 #include <algorithm>
 #include <mutex>
 
@@ -62,8 +61,8 @@ extern "C" hpt_status hpt_step_static(hpt_system s, int64_t p, const hpt_paths* 
   if (s->proj) { set_error("hpt_step_static: the projective form is not supported"); return HPT_ENOTSUP; }
   const int n = s->n;
   const size_t cs = s->prec == HPT_FP64 ? 16 : 8;
-  // layout: [re-solve counter, 256 B][re-solve list, p int64][extended
-  // Jacobian of ceil(p/128)*128 paths]; max_p bounds 511 + 8p + (p+127) B
+  // the extended Jacobian of ceil(p/128)*128 paths; max_p bounds 511 + 8p +
+  // (p+127) B, the limit that callers know (8 bytes a path more than needed)
   const size_t per_path = (size_t)n * (n + 2) * cs + sizeof(int64_t);
   const size_t jac = (size_t)n * (n + 2) * cs;
   const int64_t max_p = (int64_t)((kStaticScratchBytes - 511 - 127 * jac) / per_path);
@@ -88,9 +87,7 @@ extern "C" hpt_status hpt_step_static(hpt_system s, int64_t p, const hpt_paths* 
   // rounds of at most kChunk paths, as hpt_step runs them, so that no launch
   // is larger than the ones hpt_step makes; the scratch holds one round
   const int64_t chunk = std::min<int64_t>(p, kChunk);
-  int32_t* redo_count = (int32_t*)base;
-  int64_t* redo_list = (int64_t*)((char*)base + 256);
-  void* ext = (char*)base + 256 + ((size_t)chunk * sizeof(int64_t) + 255) / 256 * 256;
+  void* ext = base;
   cudaStream_t st = (cudaStream_t)stream;
   for (int r = 0; r < nsteps; ++r) {
     for (int64_t q0 = 0; q0 < p; q0 += chunk) {
@@ -111,8 +108,6 @@ extern "C" hpt_status hpt_step_static(hpt_system s, int64_t p, const hpt_paths* 
       a.st = sub;
       a.prm = *prm;
       a.err = s->d_err;
-      a.redo_count = redo_count;
-      a.redo_list = redo_list;
       e = launch_solve_update(s, a, st);
       if (e != cudaSuccess) {
         set_error("solve launch: %s", cudaGetErrorString(e));
