@@ -316,6 +316,11 @@ cudaError_t enqueue_round(hpt_batch_s* b, const Problem& q, const hpt_params& pr
   pm.npos = ctl;
   pm.nmax = b->nmax;
   pm.sys_tab = b->d_tab;
+  // one shape bucket: the round is a chain (each launch sets up under the tail
+  // of the one before); several: its solves are branches
+  int buckets = 0;
+  for (int bk = 0; bk < kBuckets; ++bk) buckets += q.cap_bucket[bk] > 0;
+  pm.chained = buckets == 1;
   int32_t nk = 0;
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < b->tune.steps_per_round && e == cudaSuccess; ++k) {

@@ -236,6 +236,7 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
   __shared__ float tau_f[32];
   __shared__ double tinv[32];
   __shared__ int64_t spath[32];
+  grid_wait();
   int64_t base = (int64_t)blockIdx.x * 32;
   int nmax = S.nv;
   if (MAP) {
@@ -391,9 +392,8 @@ cudaError_t launch_fx(const Fp64Sys& f, int nvs, int neq, int64_t p, const doubl
     cudaError_t e = cudaFuncSetAttribute(eval_fx_kernel<MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, fx_smem(kMaxN, true));
     if (e != cudaSuccess) return e;
   }
-  eval_fx_kernel<MAP><<<dim3((unsigned)tiles, (unsigned)fx_groups(tiles, neq)), 128, smem, st>>>(
-      f, p, y, tau, tau_is_t, ext, H, Hy, Ht, pm, tab, nvs);
-  return cudaGetLastError();
+  return launch_chained(eval_fx_kernel<MAP>, dim3((unsigned)tiles, (unsigned)fx_groups(tiles, neq)), 128, smem, st,
+                        ext != nullptr, f, p, y, tau, tau_is_t, ext, H, Hy, Ht, pm, tab, nvs);
 }
 
 }  // namespace

@@ -151,6 +151,7 @@ eval_pipe_kernel(PipeArgs P, const float2* __restrict__ y, const double* __restr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   const uint32_t tbase = *tslot;
   // tensor-memory columns: the W ring (Re MP, Im MP each), then the J ring
   auto tw_col = [&](int b) { return tbase + (uint32_t)(b * 2 * S.MP); };
@@ -424,9 +425,10 @@ cudaError_t launch_eval_pipe(hpt_system prof, const MixedSys& s, int64_t p, cons
   const int64_t grid = std::min<int64_t>(units, num_sms);
   if (grid < 1) return cudaSuccess;
   int pi = prof_begin(prof, "eval_pipe_tc", st);
-  eval_pipe_kernel<<<(unsigned)grid, kPipeThreads, smem, st>>>(a, (const float2*)y, tau, chunks, (float2*)ext, err);
+  e = launch_chained(eval_pipe_kernel, (unsigned)grid, kPipeThreads, smem, st, true, a, (const float2*)y, tau, chunks,
+                     (float2*)ext, err);
   prof_end(prof, pi, st);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace hpt

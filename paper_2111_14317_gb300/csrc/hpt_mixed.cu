@@ -84,6 +84,7 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
   uint32_t* tslot = (uint32_t*)(sm + P.s_bar + 64);
   int* sAbort = (int*)(sm + P.s_bar + 68);
 
+  grid_wait();
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = tid & 127;          // point of the tile = TMEM lane
   const int half = tid >> 7;          // warpgroup: splits the column chunks
@@ -525,11 +526,10 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
   }
   if (grid < 1) return cudaSuccess;
   int pi = prof_begin(prof, "eval_mixed_tc", st);
-  kern<<<(unsigned)grid, kEvalThreads, best_smem, st>>>(best, (const float2*)y, tin, tau_is_t, chunks,
-                                                       (float2*)out.ext, (float2*)out.H, (float2*)out.Hy,
-                                                       (float2*)out.Ht, err, pm);
+  e = launch_chained(kern, (unsigned)grid, kEvalThreads, best_smem, st, out.ext && pm.chained, best, (const float2*)y, tin, tau_is_t,
+                     chunks, (float2*)out.ext, (float2*)out.H, (float2*)out.Hy, (float2*)out.Ht, err, pm);
   prof_end(prof, pi, st);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

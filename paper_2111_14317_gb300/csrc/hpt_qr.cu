@@ -504,6 +504,7 @@ __global__ void __launch_bounds__(kQrThreads, (sizeof(T) == 4 && R == 3 && CM ==
 qr_kernel(int n, int nv, int proj, int64_t p, const void* __restrict__ ext, const void* __restrict__ yin,
           void* __restrict__ dE, void* __restrict__ dN, int32_t* __restrict__ okout, hpt_paths S, hpt_params prm) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   const int lane = threadIdx.x & (G - 1);
   const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int32_t status = path < p ? (STEP ? S.status[path] : HPT_PATH_ACTIVE) : -1;
@@ -552,6 +553,7 @@ null64_kernel(int n, int nv, int proj, int64_t p, const double2* __restrict__ ex
               double2* __restrict__ dE, double2* __restrict__ dN, int32_t* __restrict__ okout, hpt_paths S,
               hpt_params prm) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   constexpr int P = lu64_paths<G>();
   const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
   const int64_t q0 = (int64_t)blockIdx.x * P;
@@ -671,10 +673,10 @@ cudaError_t launch_qr_shape(hpt_system s, int64_t p, const void* ext, const void
   const int64_t blocks = (p * G + kQrThreads - 1) / kQrThreads;
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
   int pi = prof_begin(s, STEP ? "qr_step" : "qr_directions", st);
-  qr_kernel<T, G, R, CM, STEP><<<(unsigned)blocks, kQrThreads, smem, st>>>(s->n, s->nv, s->proj, p, ext, y, dE, dN,
-                                                                          ok, S, prm);
+  e = launch_chained(qr_kernel<T, G, R, CM, STEP>, (unsigned)blocks, kQrThreads, smem, st, true, s->n, s->nv, s->proj, p,
+                     ext, y, dE, dN, ok, S, prm);
   prof_end(s, pi, st);
-  return cudaGetLastError();
+  return e;
 }
 
 template <int G, int R, bool STEP>
@@ -685,10 +687,10 @@ cudaError_t launch_null64(hpt_system s, int64_t p, const void* ext, const void* 
   const int64_t blocks = (p + lu64_paths<G>() - 1) / lu64_paths<G>();
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
   int pi = prof_begin(s, STEP ? "qr_step" : "qr_directions", st);
-  null64_kernel<G, R, STEP><<<(unsigned)blocks, kLuThreads, lu64_smem<G>(s->nv), st>>>(
-      s->n, s->nv, s->proj, p, (const double2*)ext, (const double2*)y, (double2*)dE, (double2*)dN, ok, S, prm);
+  e = launch_chained(null64_kernel<G, R, STEP>, (unsigned)blocks, kLuThreads, lu64_smem<G>(s->nv), st, true, s->n, s->nv,
+                     s->proj, p, (const double2*)ext, (const double2*)y, (double2*)dE, (double2*)dN, ok, S, prm);
   prof_end(s, pi, st);
-  return cudaGetLastError();
+  return e;
 }
 
 // Shapes by N = nv: FP64 as the LU solves (lu_shape); FP32 reflectors (CM >=

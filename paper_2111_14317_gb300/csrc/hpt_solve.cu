@@ -633,6 +633,7 @@ __global__ void __launch_bounds__(kSolveThreads)
 solve_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
                     const __grid_constant__ hpt_params prm, int ws) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int32_t status = path < p ? S.status[path] : -1;
   const bool valid = status == HPT_PATH_ACTIVE;
@@ -919,6 +920,7 @@ __global__ void __launch_bounds__(kSolveThreads, R == 1 ? 6 : 4)
 gj_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
                  const __grid_constant__ hpt_params prm) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int32_t status = path < p ? S.status[path] : -1;
   if (!__any_sync(0xffffffffu, status == HPT_PATH_ACTIVE)) return;   // warp-uniform exit
@@ -937,6 +939,7 @@ __global__ void __launch_bounds__(kSolveThreads, R == 1 ? 6 : 4)
 gj_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
                      const __grid_constant__ hpt_params prm, PathMap pm) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   constexpr int per_warp = 32 / G;
   const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
@@ -966,6 +969,7 @@ solve_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const
                         const __grid_constant__ hpt_params prm, PathMap pm, int ws) {
   typedef float T;
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   constexpr int per_warp = 32 / G;
   const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
@@ -1014,6 +1018,7 @@ template <int G, int R>
 __global__ void __launch_bounds__(kLuThreads)
 step_fp64_kernel(int n, int64_t p, const double2* __restrict__ ext, hpt_paths S, hpt_params prm) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   constexpr int P = lu64_paths<G>();
   const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
   const int64_t q0 = (int64_t)blockIdx.x * P;
@@ -1055,6 +1060,7 @@ __global__ void __launch_bounds__(kLuThreads)
 newton_kernel(int n0, int64_t p, const double2* __restrict__ ext, double2* __restrict__ x,
               int32_t* __restrict__ done, float* __restrict__ last, double tol, PathMap pm) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   constexpr int P = lu64_paths<G>();
   const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
   const int64_t q0 = (int64_t)blockIdx.x * P + (MAP ? (int64_t)*pm.pos_begin : 0);
@@ -1340,9 +1346,8 @@ cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
   const int smem = (kSolveThreads / 32) * ws;
   cudaError_t e = set_smem(solve_update_map_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
-  solve_update_map_kernel<G, R><<<solve_grid(a.p, G), kSolveThreads, smem, st>>>(a.n, a.p, (const float2*)a.ext, a.st,
-                                                                                  a.prm, pm, ws);
-  return cudaGetLastError();
+  return launch_chained(solve_update_map_kernel<G, R>, solve_grid(a.p, G), kSolveThreads, smem, st, pm.chained, a.n, a.p,
+                        (const float2*)a.ext, a.st, a.prm, pm, ws);
 }
 
 // FP32 Gauss-Jordan solve + update (n <= 16: (G, R) = (8, 1) or (8, 2)), one
@@ -1353,17 +1358,15 @@ cudaError_t launch_gj(const StepArgs& a, cudaStream_t st) {
   if (!a.map.list) {
     cudaError_t e = set_smem(gj_update_kernel<G, R>, smem);
     if (e != cudaSuccess) return e;
-    gj_update_kernel<G, R><<<blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st>>>(
-        a.n, a.p, (const float2*)a.ext, a.st, a.prm);
-    return cudaGetLastError();
+    return launch_chained(gj_update_kernel<G, R>, blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st, true, a.n,
+                          a.p, (const float2*)a.ext, a.st, a.prm);
   }
   cudaError_t e = set_smem(gj_update_map_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
-  gj_update_map_kernel<G, R><<<solve_grid(a.p, G), kSolveThreads, smem, st>>>(
-      a.n, a.p, (const float2*)a.ext, a.st, a.prm, pm);
-  return cudaGetLastError();
+  return launch_chained(gj_update_map_kernel<G, R>, solve_grid(a.p, G), kSolveThreads, smem, st, pm.chained, a.n, a.p,
+                        (const float2*)a.ext, a.st, a.prm, pm);
 }
 
 template <int G, int R>
@@ -1371,9 +1374,8 @@ cudaError_t launch_step64_shape(const StepArgs& a, cudaStream_t st) {
   const int smem = lu64_smem<G>(a.n);
   cudaError_t e = set_smem(step_fp64_kernel<G, R>, lu64_smem<G>(G * R));
   if (e != cudaSuccess) return e;
-  step_fp64_kernel<G, R><<<blocks_for(a.p, lu64_paths<G>()), kLuThreads, smem, st>>>(
-      a.n, a.p, (const double2*)a.ext, a.st, a.prm);
-  return cudaGetLastError();
+  return launch_chained(step_fp64_kernel<G, R>, blocks_for(a.p, lu64_paths<G>()), kLuThreads, smem, st, true, a.n, a.p,
+                        (const double2*)a.ext, a.st, a.prm);
 }
 
 template <int G, int R>
@@ -1384,12 +1386,10 @@ cudaError_t launch_newton_shape(int n, int64_t p, const void* ext, void* x, int3
                      : set_smem(newton_kernel<G, R, false>, lu64_smem<G>(G * R));
   if (e != cudaSuccess) return e;
   const unsigned nb = blocks_for(p, lu64_paths<G>());
-  if (pm)
-    newton_kernel<G, R, true><<<nb, kLuThreads, smem, st>>>(n, p, (const double2*)ext, (double2*)x, done, last, tol, *pm);
-  else
-    newton_kernel<G, R, false><<<nb, kLuThreads, smem, st>>>(n, p, (const double2*)ext, (double2*)x, done, last, tol,
-                                                             PathMap());
-  return cudaGetLastError();
+  return pm ? launch_chained(newton_kernel<G, R, true>, nb, kLuThreads, smem, st, true, n, p, (const double2*)ext,
+                             (double2*)x, done, last, tol, *pm)
+            : launch_chained(newton_kernel<G, R, false>, nb, kLuThreads, smem, st, true, n, p, (const double2*)ext,
+                             (double2*)x, done, last, tol, PathMap());
 }
 
 cudaError_t launch_newton(int n, int64_t p, const void* ext, void* x, int32_t* done, float* last, double tol,
@@ -1437,9 +1437,8 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
     const int ws = warp_smem(GroupSmem<float, 32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
     e = set_smem(solve_update_kernel, smem);
     if (e != cudaSuccess) return e;
-    solve_update_kernel<<<blocks_for(a.p, kSolveThreads / 32), kSolveThreads, smem, st>>>(
-        a.n, a.p, (const float2*)a.ext, a.st, a.prm, ws);
-    e = cudaGetLastError();
+    e = launch_chained(solve_update_kernel, blocks_for(a.p, kSolveThreads / 32), kSolveThreads, smem, st, true, a.n, a.p,
+                       (const float2*)a.ext, a.st, a.prm, ws);
   }
   prof_end(s, pi, st);
   return e;
