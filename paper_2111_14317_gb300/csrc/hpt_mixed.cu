@@ -1,9 +1,9 @@
 // Mixed-precision evaluation of the homotopy and its extended Jacobian on the
 // fifth-generation tensor cores (tcgen05, accumulators in tensor memory).
 //
-// Algorithm 2 (Section 5) for tiles of 128 points: a persistent CTA of 256
-// threads walks its tiles; point r of a tile is tensor-memory lane r, served
-// by thread r of each of the two warpgroups, which split the columns:
+// Algorithm 2 (Section 5) for tiles of 128 points: a persistent CTA of two
+// or four warpgroups walks its tiles; point r of a tile is tensor-memory lane
+// r, served by thread r of each warpgroup; the warpgroups split the columns:
 //   op. 1   z = log y in FP32 (principal branch) in the units of the
 //           exponential, Re z = log2 |y|, Im z = arg y / (2 pi); Re z and
 //           Im z each split into three BF16 parts (hi + mid + lo carries the
@@ -52,12 +52,18 @@ struct MixedArgs {
   int wbuf;   // exponent accumulators W in tensor memory: 2 (next GEMM under the epilogue) or 1
   // shared-memory carve-up (bytes from the 1024-aligned base)
   int s_are, s_aim, s_invy, s_achi, s_aclo, s_const0, s_const1, s_cpart, s_bar;
+  int s_tau;  // (tau / D) log2(e) of the tile's points
   int s_zq;   // fixed angles of the tile's points ([j][128] uint32) when a system has large exponents
   int64_t p;
   int ntiles;
 };
 
-constexpr int kEvalThreads = 256;   // two warpgroups over the 128 TMEM lanes
+// Warpgroups of a CTA, each with all 128 points and its share of the columns:
+// two where two CTAs fit on an SM, four where one does (large shapes; eight
+// warps per SM left the epilogues' chains uncovered: n = 24, 54 monomials per
+// equation, 20,011 points 183 -> 178 us, and 169 with tau formed once per
+// point).
+inline int warpgroups(int ctas_per_sm) { return ctas_per_sm >= 2 ? 2 : 4; }
 
 // Barriers in shared memory: [0], [1] constant buffers; [2], [3] exponent
 // accumulators W[0], W[1]; [4] coefficient accumulator J; [5] coefficient
@@ -67,8 +73,9 @@ constexpr int kEvalThreads = 256;   // two warpgroups over the 128 TMEM lanes
 // SPLIT: the constant buffers hold only the exponent parts; the coefficient
 // part has a buffer of its own (large shapes; a compile-time choice, so that
 // the other form carries none of its code).
-template <bool MAP, bool SPLIT>
-__global__ void __launch_bounds__(kEvalThreads, 2)
+// WG: warpgroups over the 128 points, 2 or 4.
+template <bool MAP, bool SPLIT, int WG>
+__global__ void __launch_bounds__(128 * WG, WG == 2 ? 2 : 1)
 eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __restrict__ tin, int tau_is_t,
                   const uint8_t* __restrict__ chunks, float2* __restrict__ ext, float2* __restrict__ oH,
                   float2* __restrict__ oHy, float2* __restrict__ oHt, int32_t* __restrict__ err, PathMap pm_in) {
@@ -91,48 +98,67 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
   const int ntiles = pm.npos ? (*pm.npos + 127) / 128 : P.ntiles;
   // A CTA's work items are (tile, range of equations) pairs; the evaluation
   // of one (tile, equation) is the same whichever CTA does it.  Many
-  // systems: whole tiles, strided over the grid, or, when the tiles left are
-  // at most half the CTAs, `parts` CTAs per tile, each a contiguous part of
-  // its equations (a tile's equations are a serial chain of a few
-  // microseconds each: the tracks of 4,096 paths of 16 systems, n up to 24, with
-  // 32 of 152 SMs working took 63 ms and take 29.6, the concurrent solves included).  One system: the sequence
+  // systems with many tiles: whole tiles, strided over the grid.  One system,
+  // or no more tiles than CTAs (and threads, for the scan below): the sequence
   // of (tile, equation) units, tile-major, is cut into gridDim.x contiguous
   // ranges of equal length (to within one unit), so every CTA does the same
   // work whether the tiles outnumber the CTAs or not; a range that crosses
   // tile boundaries is one item per tile it touches.
-  const int64_t units = MAP ? 0 : (int64_t)ntiles * P.sys.ne;
+  // With few tiles a tile's equations would otherwise be a serial chain in one
+  // CTA (16 systems x 256 paths, n up to 24: 32 of 152 SMs at work, 63 ms a
+  // track; every tile in equal parts 29.0, equal units 26.6).
+  int* first_unit = (int*)sAcHi;   // of every tile, few-tiles form (before the E operand's first use)
+  const bool few = MAP && ntiles <= (int)gridDim.x && ntiles <= 128 * WG;
+  if (MAP && few) {
+    int* wsum = first_unit + 128 * WG + 1;
+    int v = tid < ntiles ? pm.sys_tab[pm.tile_sys[tid]].ne : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int w = __shfl_up_sync(0xffffffffu, v, o);
+      if ((tid & 31) >= o) v += w;
+    }
+    if ((tid & 31) == 31) wsum[warp] = v;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) v += wsum[w];
+    first_unit[tid + 1] = v;
+    if (tid == 0) first_unit[0] = 0;
+    __syncthreads();
+  }
+  const int64_t units = MAP ? (few ? first_unit[ntiles] : 0) : (int64_t)ntiles * P.sys.ne;
   const int64_t u0 = (int64_t)blockIdx.x * units / (int64_t)gridDim.x;
   const int64_t u1 = ((int64_t)blockIdx.x + 1) * units / (int64_t)gridDim.x;
-  const int t0 = MAP ? 0 : (int)(u0 / P.sys.ne);
-  const int parts = MAP && ntiles > 0 ? max(1, (int)gridDim.x / ntiles) : 1;
-  const int my_tiles = MAP ? (parts > 1 ? ((int)blockIdx.x < ntiles * parts ? 1 : 0)
-                                        : (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x)
-                           : (u1 > u0 ? (int)((u1 - 1) / P.sys.ne) - t0 + 1 : 0);
+  auto tile_of_unit = [&](int64_t u) {   // the last tile that begins at or before u
+    if (!MAP) return (int)(u / P.sys.ne);
+    int lo = 0, hi = ntiles - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) / 2;
+      if (first_unit[mid] <= u) lo = mid;
+      else hi = mid - 1;
+    }
+    return lo;
+  };
+  const int t0 = MAP && !few ? 0 : tile_of_unit(u0);
+  const int64_t base0 = MAP && few ? first_unit[t0] : 0;
+  const int my_tiles = MAP && !few ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
+                                   : (u1 > u0 ? tile_of_unit(u1 - 1) - t0 + 1 : 0);
   if (my_tiles <= 0) return;
   const bool lookahead = P.nbuf == 2 && P.wbuf == 2;
   const int nmax = pm.nmax ? pm.nmax : P.sys.n;
-  auto tile_of = [&](int it) {
-    return MAP ? (parts > 1 ? (int)blockIdx.x / parts : (int)blockIdx.x + it * (int)gridDim.x) : t0 + it;
-  };
+  auto tile_of = [&](int it) { return MAP && !few ? (int)blockIdx.x + it * (int)gridDim.x : t0 + it; };
   auto sys_of = [&](int tile) { return pm.tile_sys ? pm.tile_sys[tile] : 0; };
   // equations [kb, ke) of work item it (ln: the tile's equation count)
   auto krange = [&](int it, int ln, int& kb, int& ke) {
-    if (MAP) {
-      const int part = parts > 1 ? (int)blockIdx.x % parts : 0;
-      kb = ln * part / parts;
-      ke = ln * (part + 1) / parts;
+    if (MAP && !few) {
+      kb = 0;
+      ke = ln;
       return;
     }
-    const int64_t base = (int64_t)tile_of(it) * ln;
+    int64_t base = MAP ? base0 : (int64_t)tile_of(it) * ln;
+    if (MAP)   // a range of a few units: seldom beyond its second tile
+      for (int i = 0; i < it; ++i) base += pm.sys_tab[pm.tile_sys[t0 + i]].ne;
     kb = (int)(u0 > base ? u0 - base : 0);
     ke = (int)(u1 - base < (int64_t)ln ? u1 - base : (int64_t)ln);
   };
-
-  if (MAP) {   // more parts than equations: some are empty
-    int kb, ke;
-    krange(0, pm.sys_tab[sys_of(tile_of(0))].ne, kb, ke);
-    if (kb >= ke) return;
-  }
 
   if (tid == 0) {
     // 2, 3 (W full) and 4 (J full): warps 0 and 1 commit
@@ -236,12 +262,15 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
     const size_t vbase = !live ? 0 : (pm.vofs ? (size_t)pm.vofs[path] : (size_t)path * n);
     const float inv_D = S.inv_D;
     // ---- op. 1: z = log y, three-way BF16 split, 1/y (variables split by half)
+    // tau in FP64 (a warp's logarithm or exponential takes the FP64 pipe of the
+    // SM some 500 cycles): once per point, by the first warpgroup; 1/t only for
+    // the caller's H_t
+    float* sTau = (float*)(sm + P.s_tau);   // [128] (tau / D) log2(e)
     const double tv = (live && tin) ? tin[path] : (tau_is_t ? 1.0 : 0.0);
-    const double tau = tau_is_t ? log(tv) : tv;
-    const float tau2 = (float)(tau * (double)inv_D * 1.4426950408889634);   // (tau / D) log2(e)
-    const float t_inv = (float)(tau_is_t ? 1.0 / tv : exp(-tau));
+    if (half == 0) sTau[row] = (float)((tau_is_t ? log(tv) : tv) * (double)inv_D * 1.4426950408889634);
+    const float t_inv = oHt ? (float)(tau_is_t ? 1.0 / tv : exp(-tv)) : 0.f;
     uint32_t* sZq = (uint32_t*)(sm + P.s_zq);
-    for (int j = half; j < n; j += 2) {
+    for (int j = half; j < n; j += WG) {
       float2 v = live ? y[vbase + j] : make_float2(1.f, 0.f);
       float zr, zi;
       log_coords(v, zr, zi);
@@ -260,23 +289,24 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
         rem_i -= bf16_f(hi);
       }
     }
-    for (int q = 3 * n + half; q < S.KX; q += 2) {
+    for (int q = 3 * n + half; q < S.KX; q += WG) {
       *(uint16_t*)(sAre + canon(row, q, S.KX)) = 0;
       *(uint16_t*)(sAim + canon(row, q, S.KX)) = 0;
     }
     proxy_fence();
     tc_fence_before();
     __syncthreads();
+    const float tau2 = sTau[row];
     if (warp < 2 && lookahead && !issue_exp(g, S)) atomicExch(sAbort, 1);
 
     // row kk of the outputs from J: 8-column chunks (4 complex entries)
-    // alternate between the warpgroups (NJ is a multiple of 16)
+    // alternate between the warpgroups
     auto write_row = [&](int kk) {
       const uint32_t tj = t_j + lane_base;
       // the step scratch row [D_z h_kk | D_tau h_kk | h_kk] is contiguous in u
       // with stride 128 (ext_index); the solve applies diag(1/y)
       float2* erow = ext ? ext + ext_index(pos, kk, 0, nmax) : nullptr;
-      for (int c0 = 8 * half; c0 < S.NJ; c0 += 16) {
+      for (int c0 = 8 * half; c0 < S.NJ; c0 += 8 * WG) {
         float jr[8];
         tmem_ld8_j(tj + c0, S.NJ, S.jst != 0, jr);
         if (!live) continue;
@@ -317,9 +347,8 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
       {
         const float* texp = (const float*)(cbuf(g) + S.off_texp);
         const uint32_t tw = tbase + (uint32_t)((P.wbuf == 2 ? (g & 1) : 0) * 2 * S.MP) + lane_base;
-        // chunks of 8 monomials alternate between the warpgroups (MP is a
-        // multiple of 16, so both get the same number)
-        for (int c0 = 8 * half; c0 < S.MP; c0 += 16) {
+        // chunks of 8 monomials alternate between the warpgroups
+        for (int c0 = 8 * half; c0 < S.MP; c0 += 8 * WG) {
           uint32_t wre[8], wim[8];
           tmem_ld8(tw + c0, wre);
           tmem_ld8(tw + S.MP + c0, wim);
@@ -433,9 +462,12 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
                         int32_t* err, const PathMap& pm, int ctas_per_sm, cudaStream_t st) {
   if (ntiles > 0x7fffffff) return cudaErrorInvalidValue;
   const bool map = pm.list != nullptr;
-  auto pick = [map](bool split) {
-    return map ? (split ? eval_mixed_kernel<true, true> : eval_mixed_kernel<true, false>)
-               : (split ? eval_mixed_kernel<false, true> : eval_mixed_kernel<false, false>);
+  auto pick = [map](bool split, int wg) {
+    if (wg == 4)
+      return map ? (split ? eval_mixed_kernel<true, true, 4> : eval_mixed_kernel<true, false, 4>)
+                 : (split ? eval_mixed_kernel<false, true, 4> : eval_mixed_kernel<false, false, 4>);
+    return map ? (split ? eval_mixed_kernel<true, true, 2> : eval_mixed_kernel<true, false, 2>)
+               : (split ? eval_mixed_kernel<false, true, 2> : eval_mixed_kernel<false, false, 2>);
   };
   int dev = 0, max_smem = 0, sm_smem = 0;
   cudaGetDevice(&dev);
@@ -486,15 +518,16 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
     a.s_const0 = take(cbytes);
     a.s_const1 = a.nbuf == 2 ? take(cbytes) : a.s_const0;
     a.s_cpart = a.split ? take(cpart) : a.s_const0;
-    a.s_bar = take(128);
+    a.s_bar = take(128 + 512);   // one kilobyte either way
+    a.s_tau = a.s_bar + 128;
     a.p = p;
     a.ntiles = (int)ntiles;
     const int smem = off + 1024;   // slack for aligning the dynamic base
     if (smem > max_smem) continue;
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, pick(a.split));
+    e = cudaFuncGetAttributes(&fa, pick(a.split, 2));
     if (e != cudaSuccess) return e;
-    const int regs_per_cta = (fa.numRegs + 7) / 8 * 8 * kEvalThreads;
+    const int regs_per_cta = (fa.numRegs + 7) / 8 * 8 * 256;
     // 1 KB of shared memory per CTA is reserved by the system
     const int per_sm = std::min({sm_smem / (smem + 1024), 65536 / regs_per_cta, 512 / a.tmem_cols});
     if (per_sm >= 1) {
@@ -505,10 +538,11 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
     }
   }
   if (best_per_sm < 1) return cudaErrorInvalidConfiguration;
-  auto kern = pick(best.split);
+  const int per_sm = ctas_per_sm > 0 ? std::min(ctas_per_sm, best_per_sm) : best_per_sm;
+  const int wg = warpgroups(per_sm);
+  auto kern = pick(best.split, wg);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, best_smem);
   if (e != cudaSuccess) return e;
-  const int per_sm = ctas_per_sm > 0 ? std::min(ctas_per_sm, best_per_sm) : best_per_sm;
   const int64_t slots = (int64_t)num_sms() * per_sm;
   // One system: the (tile, equation) units are shared out in equal
   // contiguous ranges (see the kernel), so with few tiles a tile's equations
@@ -526,7 +560,7 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
   }
   if (grid < 1) return cudaSuccess;
   int pi = prof_begin(prof, "eval_mixed_tc", st);
-  e = launch_chained(kern, (unsigned)grid, kEvalThreads, best_smem, st, out.ext && pm.chained, best, (const float2*)y, tin, tau_is_t,
+  e = launch_chained(kern, (unsigned)grid, 128 * wg, best_smem, st, out.ext && pm.chained, best, (const float2*)y, tin, tau_is_t,
                      chunks, (float2*)out.ext, (float2*)out.H, (float2*)out.Hy, (float2*)out.Ht, err, pm);
   prof_end(prof, pi, st);
   return e;
