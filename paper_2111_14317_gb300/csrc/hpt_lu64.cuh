@@ -244,16 +244,19 @@ __device__ __forceinline__ cx<double> lu64_x(int n, const double2* A, const int*
   return mk<double>(scale_exp(v.x, k), scale_exp(v.y, k));
 }
 
-// The FP64 solves: (G, R) = (8, 1) for n <= 8, (8, 2) for n <= 16, (16, 2) for
-// n <= 32 where the paths fill the chip; 32 lanes a path where fewer than
-// kLuWarps warps would be in flight: a path's chain is then shorter (the
-// lanes that a step's entries do not fill cost nothing on an idle pipe).
-// Every shape gives the same bits.
+// The FP64 solves, lanes per path: 8 for n <= 16 and 16 for n <= 32 where the
+// paths fill the chip with kLuWarps warps; otherwise 16 (n <= 16) or 32, the
+// fewest that do, or 32.  More lanes make a path's chain shorter and leave
+// more of them without an entry (n = 8: 75 FP64 instructions a path with 8
+// lanes, 116 with 16, 200 with 32); below kLuWarps the chain counts (adjoint, n
+// = 8, 4,096 solutions: kernel 70 us with 32 lanes, 63 with 8, 61 with 16).
+// Shapes: 0 (8, 1), 1 (8, 2), 2 (16, 2), 3 (32, 1), 4 (16, 1), (lanes, unknowns
+// per lane).  Every shape gives the same bits.
 constexpr int64_t kLuWarps = 152 * 4 * 2;
 inline int lu_shape(int n, int64_t p) {
-  const int G = n <= 16 ? 8 : 16;
-  if (p * G < 32 * kLuWarps) return 3;
-  return n <= 8 ? 0 : (n <= 16 ? 1 : 2);
+  auto fills = [p](int G) { return p * G >= 32 * kLuWarps; };
+  if (n <= 16) return fills(8) ? (n <= 8 ? 0 : 1) : (fills(16) ? 4 : 3);
+  return fills(16) ? 2 : 3;
 }
 
 }  // namespace

@@ -707,7 +707,8 @@ cudaError_t launch_qr_any(hpt_system s, int64_t p, const void* ext, const void* 
     return sh == 0 ? launch_null64<8, 1, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
          : sh == 1 ? launch_null64<8, 2, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
          : sh == 2 ? launch_null64<16, 2, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
-                   : launch_null64<32, 1, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
+         : sh == 3 ? launch_null64<32, 1, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st)
+                   : launch_null64<16, 1, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
   }
   if (N <= 8) return launch_qr_shape<float, 8, 1, 10, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);
   if (N <= 16) return launch_qr_shape<float, 8, 2, 18, STEP>(s, p, ext, y, dE, dN, ok, S, prm, st);

@@ -1129,9 +1129,21 @@ __global__ void __launch_bounds__(kLuThreads)
 adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, const double2* __restrict__ x,
                const double2* __restrict__ gx, double2* __restrict__ contrib) {
   extern __shared__ __align__(16) unsigned char smem[];
+  grid_wait();
   constexpr int P = lu64_paths<G>();
   __shared__ ulonglong2 zsh[P][G * R];
   __shared__ float lfs[P][G * R];
+  __shared__ int64_t exp1[64], exp2[64], cs1[64][2], cs2[64][2];   // looked up per lane: L1 would serve a sector a lane
+  if (threadIdx.x < 64) {
+    const fx::Tables& T = fx::tables();
+    const int i = threadIdx.x;
+    exp1[i] = T.exp1[i];
+    exp2[i] = T.exp2[i];
+    cs1[i][0] = T.cs1[i][0];
+    cs1[i][1] = T.cs1[i][1];
+    cs2[i][0] = T.cs2[i][0];
+    cs2[i][1] = T.cs2[i][1];
+  }
   const int n = sys.n;
   const int lane = threadIdx.x & (G - 1), g = threadIdx.x / G;
   const int64_t q0 = (int64_t)blockIdx.x * P;
@@ -1170,7 +1182,6 @@ adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, c
   if (!__any_sync(0xffffffffu, valid)) return;
   const bool ok = lu64_solve<G>(n, A, colx, 1);
   if (!valid) return;
-  const fx::Tables& T = fx::tables();
   for (int k = 0, i = lane; i < M; i += G) {
     while (i >= sys.off[k] + sys.msz[k]) ++k;
     double mr, mi;
@@ -1186,8 +1197,8 @@ adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, c
         th += (uint64_t)((int64_t)a * (int64_t)z.y);
         wf = fmaf((float)a, lfs[g][j], wf);
       }
-      if (fx::exp_in_range(wf)) fx::exp_in(W, th, wf, T.exp1, T.exp2, T.cs1, T.cs2, mr, mi);
-      else fx::exp_of(W, th, wf, T.exp1, T.exp2, T.cs1, T.cs2, mr, mi);
+      if (fx::exp_in_range(wf)) fx::exp_in(W, th, wf, exp1, exp2, cs1, cs2, mr, mi);
+      else fx::exp_of(W, th, wf, exp1, exp2, cs1, cs2, mr, mi);
     } else {
       const double* ai = sys.ahat + (size_t)i * (n + 1);
       double wr = 0.0, wi = 0.0;
@@ -1210,46 +1221,51 @@ adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, c
 
 // Adjoint, part 2: gc[i] += sum over the chunk's solutions of contrib[q][i],
 // in a fixed order (the same bits on every run).  First pass: block (cb, r)
-// sums rows r, r + kAdjRowBlocks, ... of 32 consecutive columns, its 8 warps
-// each a strided subset, the warps' sums added in warp order (a warp reads 32
-// consecutive columns of one row: coalesced); second pass: every column's
-// kAdjRowBlocks partial sums added in order.
-constexpr int kAdjRowBlocks = 64;
+// takes 32 consecutive columns and the rows r, r + kAdjRowBlocks, .., its 32
+// warps each a strided subset (a warp reads 32 consecutive columns of one
+// row: coalesced) and then a tree over the warps; second pass: a tree over the
+// kAdjRowBlocks partial sums.  What bounds it is the latency of dependent FP64
+// additions (4,096 x 96 contributions: 16.6 us for the two passes, 18.6 with
+// chains of 64).
+constexpr int kAdjRowBlocks = 16;
 
-__global__ void __launch_bounds__(256) sum_columns_part_kernel(int64_t p, int M, const double2* __restrict__ contrib,
-                                                                double2* __restrict__ part) {
-  __shared__ double2 red[8][32];
+__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+
+__global__ void __launch_bounds__(1024) sum_columns_part_kernel(int64_t p, int M, const double2* __restrict__ contrib,
+                                                                 double2* __restrict__ part) {
+  __shared__ double2 red[32][33];
+  grid_wait();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + tx;
   double2 acc = make_double2(0.0, 0.0);
-  if (i < M)
-    for (int64_t q = (int64_t)blockIdx.y + (int64_t)kAdjRowBlocks * ty; q < p; q += (int64_t)kAdjRowBlocks * 8) {
-      const double2 v = contrib[(size_t)q * M + i];
-      acc.x += v.x;
-      acc.y += v.y;
-    }
+  if (i < M) {
+#pragma unroll 8
+    for (int64_t q = (int64_t)blockIdx.y + (int64_t)kAdjRowBlocks * ty; q < p; q += (int64_t)kAdjRowBlocks * 32)
+      acc = add2(acc, contrib[(size_t)q * M + i]);
+  }
   red[ty][tx] = acc;
   __syncthreads();
-  if (ty == 0 && i < M) {
-    for (int w = 1; w < 8; ++w) {
-      acc.x += red[w][tx].x;
-      acc.y += red[w][tx].y;
-    }
-    part[(size_t)blockIdx.y * M + i] = acc;
-  }
+  // the tree: column ty's 32 sums, one per lane
+  double2 v = red[tx][ty];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = add2(v, make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)));
+  const int col = blockIdx.x * 32 + ty;
+  if (tx == 0 && col < M) part[(size_t)blockIdx.y * M + col] = v;
 }
 
 __global__ void sum_columns_kernel(int M, const double2* __restrict__ part, double2* __restrict__ gc) {
+  grid_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
-  double2 acc = make_double2(0.0, 0.0);
-  for (int r = 0; r < kAdjRowBlocks; ++r) {
-    const double2 v = part[(size_t)r * M + i];
-    acc.x += v.x;
-    acc.y += v.y;
-  }
-  gc[i].x += acc.x;   // chunks of solutions are added in order
-  gc[i].y += acc.y;
+  double2 v[kAdjRowBlocks];
+#pragma unroll
+  for (int r = 0; r < kAdjRowBlocks; ++r) v[r] = part[(size_t)r * M + i];
+#pragma unroll
+  for (int o = kAdjRowBlocks / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int r = 0; r < o; ++r) v[r] = add2(v[r], v[r + o]);
+  gc[i] = add2(gc[i], v[0]);   // chunks of solutions are added in order
 }
 
 template <typename T>
@@ -1398,7 +1414,8 @@ cudaError_t launch_newton(int n, int64_t p, const void* ext, void* x, int32_t* d
   return sh == 0 ? launch_newton_shape<8, 1>(n, p, ext, x, done, last, tol, pm, st)
        : sh == 1 ? launch_newton_shape<8, 2>(n, p, ext, x, done, last, tol, pm, st)
        : sh == 2 ? launch_newton_shape<16, 2>(n, p, ext, x, done, last, tol, pm, st)
-                 : launch_newton_shape<32, 1>(n, p, ext, x, done, last, tol, pm, st);
+       : sh == 3 ? launch_newton_shape<32, 1>(n, p, ext, x, done, last, tol, pm, st)
+                 : launch_newton_shape<16, 1>(n, p, ext, x, done, last, tol, pm, st);
 }
 
 template <int G, int R>
@@ -1407,9 +1424,8 @@ cudaError_t launch_adjoint_shape(hpt_system s, int64_t p, const void* ext, const
   const int smem = lu64_smem<G>(s->n);
   cudaError_t e = set_smem(adjoint_kernel<G, R>, lu64_smem<G>(G * R));
   if (e != cudaSuccess) return e;
-  adjoint_kernel<G, R><<<blocks_for(p, lu64_paths<G>()), kLuThreads, smem, st>>>(
-      fp64_sys_of(s), p, s->M, (const double2*)ext, (const double2*)x, (const double2*)gx, (double2*)contrib);
-  return cudaGetLastError();
+  return launch_chained(adjoint_kernel<G, R>, blocks_for(p, lu64_paths<G>()), kLuThreads, smem, st, true, fp64_sys_of(s), p,
+                        s->M, (const double2*)ext, (const double2*)x, (const double2*)gx, (double2*)contrib);
 }
 
 }  // namespace
@@ -1423,7 +1439,8 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
     e = sh == 0 ? launch_step64_shape<8, 1>(a, st)
       : sh == 1 ? launch_step64_shape<8, 2>(a, st)
       : sh == 2 ? launch_step64_shape<16, 2>(a, st)
-                : launch_step64_shape<32, 1>(a, st);
+      : sh == 3 ? launch_step64_shape<32, 1>(a, st)
+                : launch_step64_shape<16, 1>(a, st);
     prof_end(s, pi, st);
     return e;
   }
@@ -1478,15 +1495,17 @@ cudaError_t launch_adjoint(hpt_system s, int64_t p, const void* ext, const void*
   cudaError_t e = shape == 0 ? launch_adjoint_shape<8, 1>(s, p, ext, x, gx, partial, st)
                 : shape == 1 ? launch_adjoint_shape<8, 2>(s, p, ext, x, gx, partial, st)
                 : shape == 2 ? launch_adjoint_shape<16, 2>(s, p, ext, x, gx, partial, st)
-                             : launch_adjoint_shape<32, 1>(s, p, ext, x, gx, partial, st);
+                : shape == 3 ? launch_adjoint_shape<32, 1>(s, p, ext, x, gx, partial, st)
+                             : launch_adjoint_shape<16, 1>(s, p, ext, x, gx, partial, st);
   prof_end(s, pi, st);
   if (e != cudaSuccess) return e;
   pi = prof_begin(s, "adjoint_sum", st);
-  sum_columns_part_kernel<<<dim3((unsigned)((s->M + 31) / 32), kAdjRowBlocks), 256, 0, st>>>(
-      p, s->M, (const double2*)partial, (double2*)part);
-  sum_columns_kernel<<<blocks_for(s->M, 128), 128, 0, st>>>(s->M, (const double2*)part, (double2*)gc);
+  e = launch_chained(sum_columns_part_kernel, dim3((unsigned)((s->M + 31) / 32), kAdjRowBlocks), 1024, 0, st, true, p, s->M,
+                     (const double2*)partial, (double2*)part);
+  if (e == cudaSuccess)
+    e = launch_chained(sum_columns_kernel, blocks_for(s->M, 32), 32, 0, st, true, s->M, (const double2*)part, (double2*)gc);
   prof_end(s, pi, st);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_paths_init(hpt_system s, int64_t p, const void* y0, double tau0,

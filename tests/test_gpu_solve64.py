@@ -1,5 +1,5 @@
 """The FP64 solve's lane-group shapes (GPU).  Few paths take 32 lanes each,
-many take 8 (n <= 16) or 16 lanes; an entry's arithmetic does not depend on
+more 16, many 8 (n <= 16) or 16 lanes; an entry's arithmetic does not depend on
 the shape, so the same paths give the same bits in a small and in a large
 call.  (The small shape's step is compared with the oracle in
 test_gpu_step.py, n = 1 .. 32.)"""
@@ -17,11 +17,11 @@ def test_shapes_give_the_same_bits(hpt, n):
     s = W.laurent_system(40 + n, n, 3 if n == 1 else 5, -2, 2, 8, nnz=min(n, 4))
     alpha = W.random_alpha(3, n, -1, 1)
     h = hpt.System.from_laurent(s, {"kind": "lower", "alpha_num": alpha.tolist(), "denom": 1}, 0)
-    big, small = 4900, 37   # 4,900 paths: 8 or 16 lanes each; 37: 32 lanes
+    big, mid, small = 4900, 2500, 37   # 8 or 16 lanes each; 16; 32
     y, t = W.random_points(n, big, n)
     prm = hpt.Params(tol_accept=1e-2)
     out = {}
-    for p in (big, small):
+    for p in (big, mid, small):
         st = h.new_state(p)
         st.y.copy_(torch.from_numpy(y[:p]))
         st.y_acc.copy_(st.y)
@@ -40,4 +40,5 @@ def test_shapes_give_the_same_bits(hpt, n):
         out[p]["gc"] = h.adjoint(torch.from_numpy(y[:p]).cuda(), gx).cpu().numpy()[:small]
     for f, v in out[small].items():
         assert np.array_equal(v, out[big][f][:small], equal_nan=True), f
+        assert np.array_equal(v, out[mid][f][:small], equal_nan=True), f
     assert (out[big]["accepts"] + out[big]["rejects"] >= 1).all()
