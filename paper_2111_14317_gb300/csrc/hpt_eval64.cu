@@ -259,7 +259,7 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
     if (tin && fin) {
       const double td = S.D == 1.0 ? tau : tau / S.D;
       w = fx::log2e_times(td);
-      tf = (float)td * 1.44269504f;
+      tf = (float)fmin(fmax(td, -1e30), 1e30) * 1.44269504f;   // finite, so that e = 0 takes nothing of it
     }
     tau_hi[threadIdx.x] = w.hi;
     tau_lo[threadIdx.x] = w.lo;
@@ -291,8 +291,8 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
     zs[j * 32 + q] = make_ulonglong2((unsigned long long)lg.l, lg.turn);
     lfs[j * 32 + q] = lg.lf;
     if (oHy) {
-      const double ir = 1.0 / (v.x * v.x + v.y * v.y);
-      iys[j * 32 + q] = make_double2(v.x * ir, -v.y * ir);
+      const double r2 = v.x * v.x + v.y * v.y;
+      iys[j * 32 + q] = make_double2(v.x / r2, -v.y / r2);
     }
   }
   __syncthreads();
