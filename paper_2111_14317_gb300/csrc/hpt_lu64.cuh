@@ -250,13 +250,16 @@ __device__ __forceinline__ cx<double> lu64_x(int n, const double2* A, const int*
 // more of them without an entry (n = 8: 75 FP64 instructions a path with 8
 // lanes, 116 with 16, 200 with 32); below kLuWarps the chain counts (adjoint, n
 // = 8, 4,096 solutions: kernel 70 us with 32 lanes, 63 with 8, 61 with 16).
+// For n > 16 the line lies at four fifths of that (step of 2,300 paths, n = 24:
+// 195 us with 32 lanes, 162 with 16; 2,000 paths, n = 18: 121 and 96; 1,500
+// paths, n = 24: 150 and 162).
 // Shapes: 0 (8, 1), 1 (8, 2), 2 (16, 2), 3 (32, 1), 4 (16, 1), (lanes, unknowns
 // per lane).  Every shape gives the same bits.
 constexpr int64_t kLuWarps = 152 * 4 * 2;
 inline int lu_shape(int n, int64_t p) {
   auto fills = [p](int G) { return p * G >= 32 * kLuWarps; };
-  if (n <= 16) return fills(8) ? (n <= 8 ? 0 : 1) : (fills(16) ? 4 : 3);
-  return fills(16) ? 2 : 3;
+  if (n > 16) return p * 16 >= 32 * (kLuWarps * 4 / 5) ? 2 : 3;
+  return fills(8) ? (n <= 8 ? 0 : 1) : (fills(16) ? 4 : 3);
 }
 
 }  // namespace
