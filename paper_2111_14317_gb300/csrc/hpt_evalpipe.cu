@@ -97,6 +97,10 @@ eval_pipe_kernel(PipeArgs P, const float2* __restrict__ y, const double* __restr
   const int n = S.n, ne = S.ne;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+  // The wait comes before the allocation below (a CTA that began under the
+  // launch before it must not hold tensor memory while that launch's CTAs may
+  // still have theirs to allocate on the same SM), the next launch after it.
+  grid_await();
   // this CTA's units [u0, u1) of the tile-major sequence of (tile, equation)
   const int64_t units = (int64_t)P.ntiles * ne;
   const int64_t u0 = (int64_t)blockIdx.x * units / (int64_t)gridDim.x;
@@ -151,7 +155,7 @@ eval_pipe_kernel(PipeArgs P, const float2* __restrict__ y, const double* __restr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  grid_wait();
+  grid_release();
   const uint32_t tbase = *tslot;
   // tensor-memory columns: the W ring (Re MP, Im MP each), then the J ring
   auto tw_col = [&](int b) { return tbase + (uint32_t)(b * 2 * S.MP); };

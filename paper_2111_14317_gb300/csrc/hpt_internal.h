@@ -149,10 +149,13 @@ struct PathMap {
 
 // Launch that lets the next kernel of the stream start its set-up while the
 // previous one drains (programmatic dependent launch).  Every kernel launched
-// so calls grid_wait() in all its threads before it touches device memory
-// that an earlier launch of the stream writes or reads, and before any exit;
-// so a grid ends after its predecessors, and the order of a stream holds
-// through any mixture with plain launches.
+// so calls grid_await() in all its threads before it touches device memory
+// that an earlier launch of the stream writes or reads, before it allocates
+// tensor memory and before any exit, and grid_release() after that allocation
+// (grid_wait() is both, for kernels without tensor memory).  So a grid ends
+// after its predecessors, the order of a stream holds through any mixture
+// with plain launches, and of two grids on an SM neither holds tensor memory
+// that the other needs in order to end.
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                   bool chained, const A&... args) {
@@ -169,17 +172,21 @@ inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 #ifdef __CUDACC__
-// Waits for the grids this one depends on; a small grid then lets the next
-// launch begin at once, a large one when its blocks end.  Blocks that start
-// beside a grid which fills the chip are packed onto the few free places
-// instead of being spread over the SMs (Euler/Newton directions, n = 8, 4,999
-// points: 95 us so, 152 us with every grid letting the next begin at once;
-// 50 steps of 250 paths, n = 14, grids of 28 and 16 blocks: 1,130 us without,
-// 804 with).
+// grid_await waits for the grids this one depends on; grid_release lets the
+// next launch begin at once if this grid is small (a large one: when its blocks
+// end).  Blocks that start beside a grid which fills the chip are packed onto
+// the few free places instead of being spread over the SMs (Euler/Newton
+// directions, n = 8, 4,999 points: 95 us so, 152 us with every grid letting the
+// next begin at once; 50 steps of 250 paths, n = 14, grids of 28 and 16 blocks:
+// 1,130 us without, 804 with).
 constexpr unsigned kSmallGrid = 76;   // half the SMs
-__device__ __forceinline__ void grid_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+__device__ __forceinline__ void grid_await() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() {
   if (gridDim.x * gridDim.y <= kSmallGrid) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_wait() {
+  grid_await();
+  grid_release();
 }
 #endif
 

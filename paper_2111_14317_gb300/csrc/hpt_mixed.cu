@@ -91,7 +91,7 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
   uint32_t* tslot = (uint32_t*)(sm + P.s_bar + 64);
   int* sAbort = (int*)(sm + P.s_bar + 68);
 
-  grid_wait();
+  grid_await();
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = tid & 127;          // point of the tile = TMEM lane
   const int half = tid >> 7;          // warpgroup: splits the column chunks
@@ -174,6 +174,7 @@ eval_mixed_kernel(MixedArgs P, const float2* __restrict__ y, const double* __res
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_release();
   const uint32_t tbase = *tslot;
   const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
 
