@@ -369,7 +369,7 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
   }
 }
 
-int fx_smem(int nvs, bool hy) { return nvs * 32 * (16 + 4 * 16 + (hy ? 16 : 0) + 4); }
+constexpr int fx_smem(int nvs, bool hy) { return nvs * 32 * (16 + 4 * 16 + (hy ? 16 : 0) + 4); }
 
 // Equation groups per tile: a block takes as many rounds of four equations as
 // still leave kFxBlocks blocks (the logarithms of a tile's points are taken
@@ -388,10 +388,8 @@ cudaError_t launch_fx(const Fp64Sys& f, int nvs, int neq, int64_t p, const doubl
   const int64_t tiles = (p + 31) / 32;
   if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
   const int smem = fx_smem(nvs, Hy != nullptr);
-  if (smem > 40 * 1024) {   // static shared memory (5 KB) counts towards the default 48 KB too
-    cudaError_t e = cudaFuncSetAttribute(eval_fx_kernel<MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, fx_smem(kMaxN, true));
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem<fx_smem(kMaxN, true)>(eval_fx_kernel<MAP>, smem);
+  if (e != cudaSuccess) return e;
   return launch_chained(eval_fx_kernel<MAP>, dim3((unsigned)tiles, (unsigned)fx_groups(tiles, neq)), 128, smem, st,
                         ext != nullptr, f, p, y, tau, tau_is_t, ext, H, Hy, Ht, pm, tab, nvs);
 }

@@ -423,7 +423,7 @@ cudaError_t launch_eval_pipe(hpt_system prof, const MixedSys& s, int64_t p, cons
   for (int q = 0; q < kEBuf; ++q) { a.s_e[q] = off; off += eb; }
   for (int q = 0; q < kCBuf; ++q) { a.s_c[q] = off; off += cbb; }
   a.s_bar = off;
-  cudaError_t e = cudaFuncSetAttribute(eval_pipe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem<kMaxSmem>(eval_pipe_kernel, smem);
   if (e != cudaSuccess) return e;
   const int64_t units = ntiles * s.ne;
   const int64_t grid = std::min<int64_t>(units, num_sms);

@@ -147,6 +147,19 @@ struct PathMap {
   bool chained = true;   // host: launch_chained (false in a graph whose round has branches)
 };
 
+// Allows a kernel the dynamic shared memory of this launch.  The attribute
+// belongs to the kernel, not to the launch, and host threads with handles of
+// their own launch the same kernel side by side: so every call sets the one
+// value kMost, the largest that any launch of the kernel asks for.
+template <int kMost, typename K>
+inline cudaError_t allow_smem(K kernel, int bytes) {
+  if (bytes > kMost) return cudaErrorInvalidValue;
+  return bytes > 40 * 1024   // static shared memory counts towards the default 48 KB too
+             ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost)
+             : cudaSuccess;
+}
+constexpr int kMaxSmem = 227 * 1024;   // a block's shared memory on this part
+
 // Launch that lets the next kernel of the stream start its set-up while the
 // previous one drains (programmatic dependent launch).  Every kernel launched
 // so calls grid_await() in all its threads before it touches device memory

@@ -29,12 +29,12 @@ constexpr int kLuThreads = 128;
 // Entries of one path's region: n rows of n + 2, padded to an odd count so
 // that the staging stores of eight neighbouring paths fall on distinct banks;
 // then the column exponents (n ints).
-__host__ __device__ inline int lu64_entries(int n) { return (n * (n + 2)) | 1; }
-__host__ __device__ inline int lu64_col_entries(int n) { return (n + 3) / 4; }   // ints, in double2 units
+__host__ __device__ constexpr int lu64_entries(int n) { return (n * (n + 2)) | 1; }
+__host__ __device__ constexpr int lu64_col_entries(int n) { return (n + 3) / 4; }   // ints, in double2 units
 template <int G>
 __host__ __device__ constexpr int lu64_paths() { return kLuThreads / G; }
 template <int G>
-inline int lu64_smem(int n) { return lu64_paths<G>() * (lu64_entries(n) + lu64_col_entries(n)) * 16; }
+constexpr int lu64_smem(int n) { return lu64_paths<G>() * (lu64_entries(n) + lu64_col_entries(n)) * 16; }
 
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 // v 2^k: exact, results below the normal range go to zero.

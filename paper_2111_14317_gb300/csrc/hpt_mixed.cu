@@ -557,7 +557,7 @@ cudaError_t launch_core(hpt_system prof, const MixedSys& sys, const MixedSys& ma
   const int per_sm = ctas_per_sm > 0 ? std::min(ctas_per_sm, best_per_sm) : best_per_sm;
   const int wg = warpgroups(per_sm);
   auto kern = pick(best.split, wg);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, best_smem);
+  e = allow_smem<kMaxSmem>(kern, best_smem);
   if (e != cudaSuccess) return e;
   const int64_t slots = (int64_t)num_sms() * per_sm;
   // One system: the (tile, equation) units are shared out in equal

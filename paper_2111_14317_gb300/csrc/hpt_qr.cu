@@ -658,17 +658,11 @@ __global__ void finish_proj_kernel(int n, int64_t p, hpt_paths S, double2* __res
   done[i] = s == HPT_PATH_CONVERGED ? 0 : 3;
 }
 
-template <typename K>
-cudaError_t qr_smem_attr(K kernel, int bytes) {
-  return bytes > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
-                           : cudaSuccess;
-}
-
 template <typename T, int G, int R, int CM, bool STEP>
 cudaError_t launch_qr_shape(hpt_system s, int64_t p, const void* ext, const void* y, void* dE, void* dN,
                             int32_t* ok, const hpt_paths& S, const hpt_params& prm, cudaStream_t st) {
-  const int smem = (kQrThreads / G) * QrSmem<T, G, R, CM>::bytes;
-  cudaError_t e = qr_smem_attr(qr_kernel<T, G, R, CM, STEP>, smem);
+  constexpr int smem = (kQrThreads / G) * QrSmem<T, G, R, CM>::bytes;
+  cudaError_t e = allow_smem<smem>(qr_kernel<T, G, R, CM, STEP>, smem);
   if (e != cudaSuccess) return e;
   const int64_t blocks = (p * G + kQrThreads - 1) / kQrThreads;
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
@@ -682,7 +676,7 @@ cudaError_t launch_qr_shape(hpt_system s, int64_t p, const void* ext, const void
 template <int G, int R, bool STEP>
 cudaError_t launch_null64(hpt_system s, int64_t p, const void* ext, const void* y, void* dE, void* dN, int32_t* ok,
                           const hpt_paths& S, const hpt_params& prm, cudaStream_t st) {
-  cudaError_t e = qr_smem_attr(null64_kernel<G, R, STEP>, lu64_smem<G>(G * R));
+  cudaError_t e = allow_smem<lu64_smem<G>(G * R)>(null64_kernel<G, R, STEP>, lu64_smem<G>(s->nv));
   if (e != cudaSuccess) return e;
   const int64_t blocks = (p + lu64_paths<G>() - 1) / lu64_paths<G>();
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;

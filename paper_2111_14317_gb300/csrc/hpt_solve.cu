@@ -620,7 +620,7 @@ __device__ __noinline__ void resolve_flagged(int G, bool flag, int n, int nmax, 
 __device__ __forceinline__ bool any_flagged(bool flag) { return __any_sync(0xffffffffu, flag); }
 // Shared memory of one warp of a solve kernel: its groups' regions, or one
 // path's FP64 matrix, whichever is larger.
-inline int warp_smem(int groups_bytes, int n) {
+constexpr int warp_smem(int groups_bytes, int n) {
   return std::max(groups_bytes, (lu64_entries(n) + lu64_col_entries(n)) * 16);
 }
 
@@ -1334,12 +1334,6 @@ inline unsigned blocks_for(int64_t threads, int bs) { return (unsigned)((threads
 // (32, 1) for n <= 32.
 inline int shape_of(int n) { return n <= 8 ? 0 : (n <= 16 ? 1 : 2); }
 
-template <typename K>
-cudaError_t set_smem(K kernel, int bytes) {
-  return bytes > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
-                           : cudaSuccess;
-}
-
 // Persistent grids: enough blocks to cover the positions once, capped at a
 // few waves of resident blocks (the kernels loop over positions).
 inline unsigned solve_grid(int64_t p, int G) {
@@ -1358,9 +1352,9 @@ template <int G, int R>
 cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
-  const int ws = warp_smem((32 / G) * GroupSmem<float, G * R>::bytes, std::min(pm.nmax, G * R));
-  const int smem = (kSolveThreads / 32) * ws;
-  cudaError_t e = set_smem(solve_update_map_kernel<G, R>, smem);
+  constexpr int groups = (32 / G) * GroupSmem<float, G * R>::bytes;
+  const int ws = warp_smem(groups, std::min(pm.nmax, G * R)), smem = (kSolveThreads / 32) * ws;
+  cudaError_t e = allow_smem<(kSolveThreads / 32) * warp_smem(groups, G * R)>(solve_update_map_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
   return launch_chained(solve_update_map_kernel<G, R>, solve_grid(a.p, G), kSolveThreads, smem, st, pm.chained, a.n, a.p,
                         (const float2*)a.ext, a.st, a.prm, pm, ws);
@@ -1370,14 +1364,14 @@ cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
 // system or a position map.
 template <int G, int R>
 cudaError_t launch_gj(const StepArgs& a, cudaStream_t st) {
-  const int smem = (kSolveThreads / G) * GjLayout<G, G * R>::bytes;
+  constexpr int smem = (kSolveThreads / G) * GjLayout<G, G * R>::bytes;
   if (!a.map.list) {
-    cudaError_t e = set_smem(gj_update_kernel<G, R>, smem);
+    cudaError_t e = allow_smem<smem>(gj_update_kernel<G, R>, smem);
     if (e != cudaSuccess) return e;
     return launch_chained(gj_update_kernel<G, R>, blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st, true, a.n,
                           a.p, (const float2*)a.ext, a.st, a.prm);
   }
-  cudaError_t e = set_smem(gj_update_map_kernel<G, R>, smem);
+  cudaError_t e = allow_smem<smem>(gj_update_map_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
@@ -1388,7 +1382,7 @@ cudaError_t launch_gj(const StepArgs& a, cudaStream_t st) {
 template <int G, int R>
 cudaError_t launch_step64_shape(const StepArgs& a, cudaStream_t st) {
   const int smem = lu64_smem<G>(a.n);
-  cudaError_t e = set_smem(step_fp64_kernel<G, R>, lu64_smem<G>(G * R));
+  cudaError_t e = allow_smem<lu64_smem<G>(G * R)>(step_fp64_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
   return launch_chained(step_fp64_kernel<G, R>, blocks_for(a.p, lu64_paths<G>()), kLuThreads, smem, st, true, a.n, a.p,
                         (const double2*)a.ext, a.st, a.prm);
@@ -1398,8 +1392,8 @@ template <int G, int R>
 cudaError_t launch_newton_shape(int n, int64_t p, const void* ext, void* x, int32_t* done, float* last,
                                 double tol, const PathMap* pm, cudaStream_t st) {
   const int smem = lu64_smem<G>(n);   // map: n bounds the range's systems
-  cudaError_t e = pm ? set_smem(newton_kernel<G, R, true>, lu64_smem<G>(G * R))
-                     : set_smem(newton_kernel<G, R, false>, lu64_smem<G>(G * R));
+  cudaError_t e = pm ? allow_smem<lu64_smem<G>(G * R)>(newton_kernel<G, R, true>, smem)
+                     : allow_smem<lu64_smem<G>(G * R)>(newton_kernel<G, R, false>, smem);
   if (e != cudaSuccess) return e;
   const unsigned nb = blocks_for(p, lu64_paths<G>());
   return pm ? launch_chained(newton_kernel<G, R, true>, nb, kLuThreads, smem, st, true, n, p, (const double2*)ext,
@@ -1422,7 +1416,7 @@ template <int G, int R>
 cudaError_t launch_adjoint_shape(hpt_system s, int64_t p, const void* ext, const void* x, const void* gx,
                                  void* contrib, cudaStream_t st) {
   const int smem = lu64_smem<G>(s->n);
-  cudaError_t e = set_smem(adjoint_kernel<G, R>, lu64_smem<G>(G * R));
+  cudaError_t e = allow_smem<lu64_smem<G>(G * R)>(adjoint_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
   return launch_chained(adjoint_kernel<G, R>, blocks_for(p, lu64_paths<G>()), kLuThreads, smem, st, true, fp64_sys_of(s), p,
                         s->M, (const double2*)ext, (const double2*)x, (const double2*)gx, (double2*)contrib);
@@ -1452,7 +1446,7 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
   } else {
     pi = prof_begin(s, "solve_update_fp32", st);
     const int ws = warp_smem(GroupSmem<float, 32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
-    e = set_smem(solve_update_kernel, smem);
+    e = allow_smem<(kSolveThreads / 32) * warp_smem(GroupSmem<float, 32>::bytes, kMaxN)>(solve_update_kernel, smem);
     if (e != cudaSuccess) return e;
     e = launch_chained(solve_update_kernel, blocks_for(a.p, kSolveThreads / 32), kSolveThreads, smem, st, true, a.n, a.p,
                        (const float2*)a.ext, a.st, a.prm, ws);

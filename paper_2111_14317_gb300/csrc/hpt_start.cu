@@ -127,10 +127,7 @@ extern "C" hpt_status hpt_binomial_start_device(int32_t n, const int32_t* msz, c
   if (blocks > 0x7fffffff) { set_error("count too large"); return HPT_ERANGE; }
   const StartDev d = device_consts(S);
   const int smem = d.nj * (d.n * 16 + kStartTile * 8);
-  cudaError_t e = cudaSuccess;
-  if (smem > 40 * 1024)
-    e = cudaFuncSetAttribute(start_points_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kMaxN * (kMaxN * 16 + kStartTile * 8));
+  cudaError_t e = allow_smem<kMaxN * (kMaxN * 16 + kStartTile * 8)>(start_points_kernel, smem);
   if (e == cudaSuccess) {
     start_points_kernel<<<(unsigned)blocks, kStartThreads, smem, (cudaStream_t)stream>>>(d, first, count,
                                                                                         (double2*)y0_dev);
