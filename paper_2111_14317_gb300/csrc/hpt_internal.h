@@ -147,6 +147,13 @@ struct PathMap {
   bool chained = true;   // host: launch_chained (false in a graph whose round has branches)
 };
 
+// The error of a call, no longer pending: the caller reports it, and the next
+// plain launch (which asks cudaGetLastError) must not.
+inline cudaError_t taken(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // Allows a kernel the dynamic shared memory of this launch.  The attribute
 // belongs to the kernel, not to the launch, and host threads with handles of
 // their own launch the same kernel side by side: so every call sets the one
@@ -154,9 +161,8 @@ struct PathMap {
 template <int kMost, typename K>
 inline cudaError_t allow_smem(K kernel, int bytes) {
   if (bytes > kMost) return cudaErrorInvalidValue;
-  return bytes > 40 * 1024   // static shared memory counts towards the default 48 KB too
-             ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost)
-             : cudaSuccess;
+  if (bytes <= 40 * 1024) return cudaSuccess;   // static shared memory counts towards the default 48 KB too
+  return taken(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost));
 }
 constexpr int kMaxSmem = 227 * 1024;   // a block's shared memory on this part
 
@@ -182,7 +188,7 @@ inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, siz
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+  return taken(cudaLaunchKernelEx(&cfg, kern, P(args)...));
 }
 #ifdef __CUDACC__
 // grid_await waits for the grids this one depends on; grid_release lets the
