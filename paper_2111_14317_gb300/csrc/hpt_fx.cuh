@@ -43,7 +43,7 @@ struct Tables {
   int64_t exp1[64];       // 2^(i/64), Q62
   int64_t exp2[64];       // 2^((j + 1/2)/4096), Q62
   int64_t cs1[64][2];     // cos, sin of i/64 revolution, Q62
-  int64_t cs2[64][2];     // cos, sin of (j + 1/2)/4096 revolution, Q62
+  int64_t cs2[64][2];     // cos, sin of j/4096 revolution, Q62
   uint64_t at[33];        // atan(i/32) in revolutions, Q64
   int64_t lat[33];        // log2 sqrt(1 + (i/32)^2), Q60
   uint32_t rcp[128];      // 1/(1 + (i + 1/2)/128), Q32
@@ -109,7 +109,7 @@ constexpr Tables make_tables() {
   for (int i = 0; i < 64; ++i) {
     t.exp1[i] = round90(exp90(kLn2_90 * (unsigned)i / 64), 62);
     t.exp2[i] = round90(exp90(kLn2_90 * (unsigned)(2 * i + 1) / 8192), 62);
-    const u128 x1 = kPi90 * (unsigned)i / 32, x2 = kPi90 * (unsigned)(2 * i + 1) / 4096;
+    const u128 x1 = kPi90 * (unsigned)i / 32, x2 = kPi90 * (unsigned)i / 2048;
     t.cs1[i][0] = cs62(x1, 0);
     t.cs1[i][1] = cs62(x1, 1);
     t.cs2[i][0] = cs62(x2, 0);
@@ -329,8 +329,11 @@ HPT_FX int64_t times(int64_t k, const Wide& w) {
   return (int64_t)((uint64_t)k * w.hi + umulhi((uint64_t)k, w.lo) - (k < 0 ? w.lo : 0));
 }
 
-// cos and sin of theta (revolutions, Q64), Q62.
+// cos and sin of theta (revolutions, Q64), Q62.  The nearest multiple of
+// 1/4096 revolution comes from the tables, so multiples of a quarter turn give
+// exactly 0 and +-1: what is real stays real.
 HPT_FX void cossin(uint64_t th, const int64_t (*cs1)[2], const int64_t (*cs2)[2], int64_t& c, int64_t& s) {
+  th += (uint64_t)1 << 51;
   const int i = (int)(th >> 58), j = (int)(th >> 52) & 63;
   const int64_t r = (int64_t)(th & (((uint64_t)1 << 52) - 1)) - ((int64_t)1 << 51);
   const int64_t c1 = cs1[i][0], s1 = cs1[i][1], c2 = cs2[j][0], s2 = cs2[j][1];

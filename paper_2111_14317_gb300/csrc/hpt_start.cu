@@ -82,7 +82,9 @@ start_points_kernel(const __grid_constant__ StartDev S, int64_t first, int64_t c
       hi += lo < pl ? 1 : 0;
     }
     int64_t c, s;
-    fx::cossin(S.turn0[r] + hi, cs1, cs2, c, s);
+    // rounded: the truncated fractions of a whole number of quarter turns lie
+    // just below it
+    fx::cossin(S.turn0[r] + hi + (lo >> 63), cs1, cs2, c, s);
     const double m = S.mag[r];
     out[e] = make_double2(m * q62_to_double(c), m * q62_to_double(s));
   }
