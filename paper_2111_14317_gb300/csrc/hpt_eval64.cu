@@ -157,19 +157,14 @@ eval_fp64_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const doub
 
 // One monomial of the fixed-point evaluation.  op. 2 of Algorithm 2: W = log c
 // + [z, tau] . A[:, i] ..
-__device__ __forceinline__ void fx_begin(const FxMono& m, const fx::Wide& tw, float tf, int64_t& W, uint64_t& th,
-                                         float& wf) {
-  W = m.lc;
-  th = m.turn;
-  wf = fmaf(m.ef, tf, m.lcf);
-  if (m.e) W += fx::times((int64_t)m.e, tw);
+__device__ __forceinline__ fx::Sum fx_begin(const FxMono& m, const fx::Wide& tw, float tf) {
+  fx::Sum s{(uint64_t)m.lc, m.turn, fmaf(m.ef, tf, m.lcf)};
+  if (m.e) s.w += fx::times((int64_t)m.e, tw);
+  return s;
 }
-__device__ __forceinline__ void fx_add(const FxEnt& e, const ulonglong2* zl, const float* ll, int64_t& W,
-                                       uint64_t& th, float& wf) {
+__device__ __forceinline__ void fx_add(const FxEnt& e, const ulonglong2* zl, const float* ll, fx::Sum& s) {
   const ulonglong2 z = zl[e.j * 32];
-  W += (int64_t)e.a * (int64_t)z.x;
-  th += (uint64_t)((int64_t)e.a * (int64_t)z.y);
-  wf = fmaf((float)e.a, ll[e.j * 32], wf);
+  fx::add_power(s, e.a, z.x, z.y, ll[e.j * 32]);
 }
 // .. and its value times (a, e/D, 1), accumulated over the equation's
 // monomials.
@@ -315,27 +310,23 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
       const FxMono m0 = S.mono[i], m1 = S.mono[i + two];
       const FxEnt* __restrict__ e0 = S.ent + m0.ent;
       const FxEnt* __restrict__ e1 = S.ent + m1.ent;
-      int64_t W0, W1;
-      uint64_t th0, th1;
-      float wf0, wf1;
-      fx_begin(m0, tw, tf, W0, th0, wf0);
-      fx_begin(m1, tw, tf, W1, th1, wf1);
+      fx::Sum s0 = fx_begin(m0, tw, tf), s1 = fx_begin(m1, tw, tf);
       const int both = min(m0.nnz, m1.nnz);
       int t = 0;
 #pragma unroll 4
       for (; t < both; ++t) {
-        fx_add(e0[t], zl, ll, W0, th0, wf0);
-        fx_add(e1[t], zl, ll, W1, th1, wf1);
+        fx_add(e0[t], zl, ll, s0);
+        fx_add(e1[t], zl, ll, s1);
       }
-      for (int u = t; u < m0.nnz; ++u) fx_add(e0[u], zl, ll, W0, th0, wf0);
-      for (int u = t; u < m1.nnz; ++u) fx_add(e1[u], zl, ll, W1, th1, wf1);
+      for (int u = t; u < m0.nnz; ++u) fx_add(e0[u], zl, ll, s0);
+      for (int u = t; u < m1.nnz; ++u) fx_add(e1[u], zl, ll, s1);
       double er0, ei0, er1, ei1;
-      if (fx::exp_in_range(wf0) && fx::exp_in_range(wf1)) {
-        fx::exp_in(W0, th0, wf0, exp1, exp2, cs1, cs2, er0, ei0);
-        fx::exp_in(W1, th1, wf1, exp1, exp2, cs1, cs2, er1, ei1);
+      if (fx::exp_in_range(s0.f) && fx::exp_in_range(s1.f)) {
+        fx::exp_in((int64_t)s0.w, s0.turn, s0.f, exp1, exp2, cs1, cs2, er0, ei0);
+        fx::exp_in((int64_t)s1.w, s1.turn, s1.f, exp1, exp2, cs1, cs2, er1, ei1);
       } else {
-        fx::exp_of(W0, th0, wf0, exp1, exp2, cs1, cs2, er0, ei0);
-        fx::exp_of(W1, th1, wf1, exp1, exp2, cs1, cs2, er1, ei1);
+        fx::exp_of((int64_t)s0.w, s0.turn, s0.f, exp1, exp2, cs1, cs2, er0, ei0);
+        fx::exp_of((int64_t)s1.w, s1.turn, s1.f, exp1, exp2, cs1, cs2, er1, ei1);
       }
       fx_accumulate(m0, e0, er0, ei0, acc, accT, accH);
       if (two) fx_accumulate(m1, e1, er1, ei1, acc, accT, accH);

@@ -325,8 +325,21 @@ HPT_FX Wide log2e_times(double t) {
   return o;
 }
 // The Q60 part of k w for an integer k.
-HPT_FX int64_t times(int64_t k, const Wide& w) {
-  return (int64_t)((uint64_t)k * w.hi + umulhi((uint64_t)k, w.lo) - (k < 0 ? w.lo : 0));
+HPT_FX uint64_t times(int64_t k, const Wide& w) {
+  return (uint64_t)k * w.hi + umulhi((uint64_t)k, w.lo) - (k < 0 ? w.lo : 0);
+}
+
+// An exponent sum: W modulo 16 (Q60) and the phase (Q64), which wrap around
+// (unsigned: in signed arithmetic that would be undefined), and W in FP32.
+struct Sum {
+  uint64_t w, turn;
+  float f;
+};
+// += a log y, for y's logarithm (l, turn, lf).
+HPT_FX void add_power(Sum& s, int32_t a, uint64_t l, uint64_t turn, float lf) {
+  s.w += (uint64_t)(int64_t)a * l;
+  s.turn += (uint64_t)(int64_t)a * turn;
+  s.f = fmaf((float)a, lf, s.f);
 }
 
 // cos and sin of theta (revolutions, Q64), Q62.  The nearest multiple of

@@ -1187,18 +1187,14 @@ adjoint_kernel(Fp64Sys sys, int64_t p, int M, const double2* __restrict__ ext, c
     double mr, mi;
     if (sys.mono) {
       const FxMono m = sys.mono[i];
-      int64_t W = 0;
-      uint64_t th = 0;
-      float wf = 0.f;
+      fx::Sum w{0, 0, 0.f};
       for (int t = 0; t < m.nnz; ++t) {
         const int a = sys.ent[m.ent + t].a, j = sys.ent[m.ent + t].j;
         const ulonglong2 z = zsh[g][j];
-        W += (int64_t)a * (int64_t)z.x;
-        th += (uint64_t)((int64_t)a * (int64_t)z.y);
-        wf = fmaf((float)a, lfs[g][j], wf);
+        fx::add_power(w, a, z.x, z.y, lfs[g][j]);
       }
-      if (fx::exp_in_range(wf)) fx::exp_in(W, th, wf, exp1, exp2, cs1, cs2, mr, mi);
-      else fx::exp_of(W, th, wf, exp1, exp2, cs1, cs2, mr, mi);
+      if (fx::exp_in_range(w.f)) fx::exp_in((int64_t)w.w, w.turn, w.f, exp1, exp2, cs1, cs2, mr, mi);
+      else fx::exp_of((int64_t)w.w, w.turn, w.f, exp1, exp2, cs1, cs2, mr, mi);
     } else {
       const double* ai = sys.ahat + (size_t)i * (n + 1);
       double wr = 0.0, wi = 0.0;
