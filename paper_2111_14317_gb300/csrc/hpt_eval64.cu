@@ -166,6 +166,23 @@ __device__ __forceinline__ void fx_add(const FxEnt& e, const ulonglong2* zl, con
   const ulonglong2 z = zl[e.j * 32];
   fx::add_power(s, e.a, z.x, z.y, ll[e.j * 32]);
 }
+// The FP32 sum of a monomial at a point with coordinates 0 or infinite (mask;
+// their log2|y| is -inf or +inf in ll), or with tau infinite: -inf (the
+// monomial is 0), or NaN where the product is not defined: a factor infinite,
+// 0 times infinity, or such a coordinate (or t) to the power 0, as
+// exp(<a, log y>) has it.
+__device__ __noinline__ float fx_special(const FxMono* __restrict__ mono, const FxEnt* __restrict__ en, uint32_t mask,
+                                         float tf, const float* ll) {
+  const FxMono m = *mono;
+  float f = m.e ? m.ef * tf : tf - tf;
+  f += m.lcf;
+  for (int t = 0; t < m.nnz; ++t) {
+    const FxEnt x = en[t];
+    f += (float)x.a * ll[x.j * 32];
+    mask &= ~(1u << x.j);
+  }
+  return mask ? __int_as_float(0x7fffffff) : f;
+}
 // .. and its value times (a, e/D, 1), accumulated over the equation's
 // monomials.
 __device__ __forceinline__ void fx_accumulate(const FxMono& m, const FxEnt* __restrict__ en, double er, double ei,
@@ -228,7 +245,8 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
   float* lfs = (float*)(iys + (oHy ? nvs * 32 : 0));
   __shared__ int64_t exp1[64], exp2[64], cs1[64][2], cs2[64][2];
   __shared__ uint64_t tau_hi[32], tau_lo[32];
-  __shared__ float tau_f[32];
+  __shared__ float tau_f[32], tau_inf[32];   // NaN in tau_f sends a point's monomials to fx_special
+  __shared__ uint32_t special[32];           // coordinates 0 or infinite
   __shared__ double tinv[32];
   __shared__ int64_t spath[32];
   grid_wait();
@@ -258,7 +276,9 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
     }
     tau_hi[threadIdx.x] = w.hi;
     tau_lo[threadIdx.x] = w.lo;
-    tau_f[threadIdx.x] = fin ? tf : __int_as_float(0x7fffffff);   // NaN: every entry of the point
+    tau_f[threadIdx.x] = fin ? tf : __int_as_float(0x7fffffff);
+    tau_inf[threadIdx.x] = fin ? tf : (float)tau;
+    special[threadIdx.x] = 0;
     if (oHt) tinv[threadIdx.x] = 1.0 / tv;   // user layout: t is given
   }
   if (threadIdx.x >= 64) {   // the last two warps stage the tables
@@ -274,15 +294,19 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
   __syncthreads();
 
   // op. 1 of Algorithm 2: Z <- log Y, and 1/y for the final diag(e^{-z})
-  // scaling.  A coordinate without a logarithm (0, infinite, NaN) makes the
-  // whole point NaN.
+  // scaling.  A coordinate without a logarithm: 0 and infinity are fx_special's
+  // (its sums are -inf or NaN), NaN makes the whole point NaN.
   for (int idx = threadIdx.x; idx < 32 * nv; idx += 128) {
     const int q = idx / nv, j = idx - q * nv;
     const int64_t path = spath[q];
     double2 v = make_double2(1.0, 0.0);
     if (path >= 0) v = y[(MAP ? (size_t)pm.vofs[path] : (size_t)path * nv) + j];
     fx::Log lg;
-    if (!fx::log_of(v.x, v.y, lg)) tau_f[q] = __int_as_float(0x7fffffff);
+    if (!fx::log_of(v.x, v.y, lg)) {
+      tau_f[q] = __int_as_float(0x7fffffff);
+      lg.lf = v.x != v.x || v.y != v.y ? __int_as_float(0x7fffffff) : (v.x == 0.0 && v.y == 0.0 ? -INFINITY : INFINITY);
+      atomicOr(&special[q], 1u << j);
+    }
     zs[j * 32 + q] = make_ulonglong2((unsigned long long)lg.l, lg.turn);
     lfs[j * 32 + q] = lg.lf;
     if (oHy) {
@@ -325,6 +349,10 @@ eval_fx_kernel(Fp64Sys S, int64_t p, const double2* __restrict__ y, const double
         fx::exp_in((int64_t)s0.w, s0.turn, s0.f, exp1, exp2, cs1, cs2, er0, ei0);
         fx::exp_in((int64_t)s1.w, s1.turn, s1.f, exp1, exp2, cs1, cs2, er1, ei1);
       } else {
+        if (tf != tf) {
+          s0.f = fx_special(S.mono + i, e0, special[lane], tau_inf[lane], ll);
+          s1.f = fx_special(S.mono + i + two, e1, special[lane], tau_inf[lane], ll);
+        }
         fx::exp_of((int64_t)s0.w, s0.turn, s0.f, exp1, exp2, cs1, cs2, er0, ei0);
         fx::exp_of((int64_t)s1.w, s1.turn, s1.f, exp1, exp2, cs1, cs2, er1, ei1);
       }
