@@ -97,16 +97,11 @@ eval_pipe_kernel(PipeArgs P, const float2* __restrict__ y, const double* __restr
   const int n = S.n, ne = S.ne;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  // The wait comes before the allocation below (a CTA that began under the
-  // launch before it must not hold tensor memory while that launch's CTAs may
-  // still have theirs to allocate on the same SM), the next launch after it.
-  grid_await();
   // this CTA's units [u0, u1) of the tile-major sequence of (tile, equation)
   const int64_t units = (int64_t)P.ntiles * ne;
   const int64_t u0 = (int64_t)blockIdx.x * units / (int64_t)gridDim.x;
   const int64_t u1 = ((int64_t)blockIdx.x + 1) * units / (int64_t)gridDim.x;
   const int U = (int)(u1 - u0);
-  if (U <= 0) return;
   const int t_first = (int)(u0 / ne);
   const int t_last = (int)((u1 - 1) / ne);
   const int k_first = (int)(u0 - (int64_t)t_first * ne);
@@ -147,6 +142,11 @@ eval_pipe_kernel(PipeArgs P, const float2* __restrict__ y, const double* __restr
     *sAbort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // The wait comes before the allocation (a CTA that began under the launch
+  // before it must not hold tensor memory while that launch's CTAs may still
+  // have theirs to allocate on the same SM), the next launch after it.
+  grid_await();
+  if (U <= 0) return;
   if (warp == kXrWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
                  "r"(P.tmem_cols));
