@@ -37,13 +37,14 @@ template <int G>
 constexpr int lu64_smem(int n) { return lu64_paths<G>() * (lu64_entries(n) + lu64_col_entries(n)) * 16; }
 
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
-// v 2^k: exact, results below the normal range go to zero.
+// v 2^k, in integers; operands and results below the normal range (and
+// overflows) go to the library's, zeros, infinities and NaN stay.
+__device__ __noinline__ double scale_far(double v, int k) { return scalbn(v, k); }
 __device__ __forceinline__ double scale_exp(double v, int k) {
-  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff, f = e + k;
-  if (e == 0 || f < 1) return 0.0;
-  if (e == 0x7ff) return v;
-  if (f >= 0x7ff) return __hiloint2double((hi & (int)0x80000000) | 0x7ff00000, 0);
-  return __hiloint2double(hi + (int)((unsigned)k << 20), __double2loint(v));
+  const int hi = __double2hiint(v), lo = __double2loint(v), e = (hi >> 20) & 0x7ff;
+  const bool in = (unsigned)(e - 1) < 0x7feu && (unsigned)(e + k - 1) < 0x7feu;
+  if (!in && e != 0x7ff && ((hi << 1) | lo) != 0) return scale_far(v, k);   // seldom, so no branch for the zeros
+  return __hiloint2double(hi + (in ? (int)((unsigned)k << 20) : 0), lo);
 }
 // FP32 copy by bit pattern (truncated; 0 below FP32's range, infinity above).
 __device__ __forceinline__ float trunc_f32(double v) {
@@ -52,8 +53,9 @@ __device__ __forceinline__ float trunc_f32(double v) {
   if (e > 1150) return __int_as_float(0x7f800000);
   return __int_as_float(((e - 896) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)__double2loint(v) >> 29));
 }
-// 1/v for a normal v, within about an ulp: the hardware's approximation and
-// two Newton steps.
+// 1/v for a normal v (and a normal 1/v): the hardware's approximation, whose
+// relative error squares in each of the two Newton steps (from about 2^-20 to
+// 2^-40 and below 2^-75), so that only the last fma's rounding is left.
 __device__ __forceinline__ double rcp_newton(double v) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
@@ -124,11 +126,12 @@ __device__ __forceinline__ bool lu64_solve(int n, double2* A, int* colx, int sig
     const int kr = m == 0 ? 0 : 1022 - m;
 #pragma unroll
     for (int t = 0; t < R; ++t) {
-      if (ex[t] + kr > 0) colmax[t] = max(colmax[t], ex[t] ? ex[t] + kr : 0);
       const int c = lane + G * t;
       if (c < n) {
         const double2 v = A[r * LD + c];
-        A[r * LD + c] = make_double2(scale_exp(v.x, kr), scale_exp(v.y, kr));
+        const double x = scale_exp(v.x, kr), y = scale_exp(v.y, kr);
+        colmax[t] = max(colmax[t], max(exp_field(x), exp_field(y)));
+        A[r * LD + c] = make_double2(x, y);
       }
     }
     if (lane < 2) {
@@ -173,8 +176,11 @@ __device__ __forceinline__ bool lu64_solve(int n, double2* A, int* colx, int sig
     __syncwarp();
     const double2 pj = A[j * LD + j];
     const double p2 = pj.x * pj.x + pj.y * pj.y;
-    if (exp_field(p2) == 0 || exp_field(p2) == 0x7ff) ok = false;
-    const double rp = rcp_newton(p2);
+    double rp = rcp_newton(p2);
+    if (exp_field(p2) == 0 || exp_field(p2) == 0x7ff) {   // seldom: the reciprocal by division while it is finite
+      rp = 1.0 / p2;
+      if (!(p2 > 0.0) || exp_field(p2) == 0x7ff || exp_field(rp) == 0x7ff) ok = false;
+    }
     const double2 inv = make_double2(pj.x * rp, -pj.y * rp);
     for (int i = j + 1 + lane; i < n; i += G) {
       const double2 v = A[i * LD + j];
