@@ -136,7 +136,7 @@ typedef struct {
                            the n = 16 throughput workload), so the default re-solves the
                            typical path whose kappa_1 exceeds about 1e6 (Section 6's remark
                            on ill-conditioned systems).  A lower bound costs time: a step of
-                           65,536 paths at n = 16 takes 0.2 ms, and 2.4 ms when every path is
+                           65,536 paths at n = 16 takes 0.2 ms, and 1.7 ms when every path is
                            re-solved */
   double eps0;          /* tau0 = ln(eps0) / s_min (smallest positive e/D), default 1e-10 */
   int32_t predictor;    /* 0 (default): Euler, y = y_acc + h dE_acc.  1: cubic Hermite, once a

@@ -578,50 +578,91 @@ __device__ __forceinline__ int64_t pm_begin(const PathMap& m) { return m.pos_beg
 
 // FP64 re-solve of the paths that a warp's FP32 solves flagged (pivot ratio
 // above prm.cond_max): same FP32 Jacobian, FP64 factorisation, then the step
-// control in the FP32 state, one path after another with all 32 lanes, in the
-// warp's own shared memory (W: lu64_entries + lu64_col_entries of n).  Flagged
-// paths are rare; a launch of their own, with its list and counter to clear,
-// cost every step 6 us whether there was one or not (250 paths, n = 14: 28.7
-// -> 22.6 us a step; 65,536 paths, n = 16: 212 -> 206 us, and with every path
-// flagged 4.2 -> 2.4 ms).  Call with the warp
-// converged; flag and the path's data are group-uniform.
+// control in the FP32 state, in the warp's own shared memory.  Flagged paths
+// are rare; a launch of their own, with its list and counter to clear, cost
+// every step 6 us whether there was one or not (250 paths, n = 14: 28.7 ->
+// 22.6 us a step; 65,536 paths, n = 16: 212 -> 206 us).
+// resolve_round: the first 32 / GS flagged groups of m (a bit for each group's
+// first lane), GS lanes each; W holds 32 / GS times lu64_entries +
+// lu64_col_entries of n; n <= GS RS.
+template <int GS, int RS>
+__device__ __noinline__ void resolve_round(unsigned m, int n, int nmax, int64_t q, int64_t path, size_t vbase,
+                                           const float2* __restrict__ ext, const hpt_paths& S, const hpt_params& prm,
+                                           double2* W) {
+  constexpr int K = 32 / GS;
+  const int l = threadIdx.x & (GS - 1), g = (threadIdx.x & 31) / GS;
+  double2* A = W + g * lu64_entries(n);
+  int* colx = (int*)(W + K * lu64_entries(n)) + g * 4 * lu64_col_entries(n);
+#pragma unroll
+  for (int k = 0; k + 1 < K; ++k)
+    if (k < g) m &= m - 1;
+  const bool act = m != 0;
+  const int src = act ? __ffs(m) - 1 : 0;
+  const int64_t qs = __shfl_sync(0xffffffffu, q, src), ps = __shfl_sync(0xffffffffu, path, src);
+  const size_t vs = __shfl_sync(0xffffffffu, (unsigned long long)vbase, src);
+  __syncwarp();   // the warp's shared memory is free
+  const int np2 = n + 2;
+  for (int e = l; act && e < n * np2; e += GS) {
+    const int k = e / np2, u = e - k * np2;
+    const float2 v = ext[ext_index(qs, k, u, nmax)];
+    A[e] = make_double2((double)v.x, (double)v.y);
+  }
+  __syncwarp();
+  const bool ok = lu64_solve<GS>(n, A, colx, -1);
+  if (act) {   // group-uniform; only group-masked shuffles
+    cx<float> fE[RS], fN[RS];
+#pragma unroll
+    for (int s = 0; s < RS; ++s) {
+      const int c = l + GS * s;
+      fE[s] = fN[s] = mk<float>(0.f, 0.f);
+      if (c < n) {
+        const cx<double> e = lu64_x(n, A, colx, c, 0), f = lu64_x(n, A, colx, c, 1);
+        fE[s] = mk<float>((float)e.x, (float)e.y);
+        fN[s] = mk<float>((float)f.x, (float)f.y);
+      }
+    }
+    update_path<float, GS, RS>(n, ps, vs, HPT_PATH_ACTIVE, ok, fE, fN, S, prm);
+  }
+  __syncwarp();
+}
+// The flagged paths of a warp, a single one with all 32 lanes, more of them 32
+// / GS at a time: their chains of dependent steps, which bound it, run side by
+// side.  us a step with every path flagged, for a launch of its own, one after
+// another in the warp, and so: n = 8, 128 paths 54, 81, 35; n = 16, 128 paths
+// 165, 178, 117, 65,536 paths 4,172, 2,426, 1,646; many systems, n = 20 and 24,
+// 128 paths 214, 263, 200 and 263, 347, 269 (a single path at n = 24: 121).
+// Call with the warp converged; flag and the path's data are uniform in the
+// groups of G lanes.
+template <int GS, int RS>
 __device__ __noinline__ void resolve_flagged(int G, bool flag, int n, int nmax, int64_t q, int64_t path, size_t vbase,
                                              const float2* __restrict__ ext, const hpt_paths& S,
                                              const hpt_params& prm, double2* W) {
-  const int lane = threadIdx.x & 31;
-  unsigned m = __ballot_sync(0xffffffffu, flag && (lane & (G - 1)) == 0);
+  unsigned m = __ballot_sync(0xffffffffu, flag && (threadIdx.x & (G - 1)) == 0);
   while (m) {
-    const int src = __ffs(m) - 1;
-    m &= m - 1;
-    const int64_t qs = __shfl_sync(0xffffffffu, q, src), ps = __shfl_sync(0xffffffffu, path, src);
-    const size_t vs = __shfl_sync(0xffffffffu, (unsigned long long)vbase, src);
-    __syncwarp();   // the warp's shared memory is free
-    const int np2 = n + 2;
-    for (int e = lane; e < n * np2; e += 32) {
-      const int k = e / np2, u = e - k * np2;
-      const float2 v = ext[ext_index(qs, k, u, nmax)];
-      W[e] = make_double2((double)v.x, (double)v.y);
+    if (GS == 32 || (m & (m - 1)) == 0) {
+      resolve_round<32, 1>(m, n, nmax, q, path, vbase, ext, S, prm, W);
+      m &= m - 1;
+    } else {
+      resolve_round<GS, RS>(m, n, nmax, q, path, vbase, ext, S, prm, W);
+#pragma unroll
+      for (int k = 0; k < 32 / GS; ++k) m &= m - 1;
     }
-    __syncwarp();
-    int* colx = (int*)(W + lu64_entries(n));
-    const bool ok = lu64_solve<32>(n, W, colx, -1);
-    cx<float> fE[1], fN[1];
-    fE[0] = fN[0] = mk<float>(0.f, 0.f);
-    if (lane < n) {
-      const cx<double> e = lu64_x(n, W, colx, lane, 0), f = lu64_x(n, W, colx, lane, 1);
-      fE[0] = mk<float>((float)e.x, (float)e.y);
-      fN[0] = mk<float>((float)f.x, (float)f.y);
-    }
-    update_path<float, 32, 1>(n, ps, vs, HPT_PATH_ACTIVE, ok, fE, fN, S, prm);
-    __syncwarp();
   }
 }
+// Lanes per re-solved path and unknowns per lane, by the FP32 solve's shape: 8
+// (four paths at once) for n <= 8, 16 for n <= 24, 32 where a warp has one path.
+template <int G, int R>
+struct Resolve {
+  static constexpr int GS = G == 32 ? 32 : (R == 1 ? 8 : 16), RS = G * R <= GS ? 1 : 2;
+};
 // Whether the warp has a flagged path at all (the usual answer is no).
 __device__ __forceinline__ bool any_flagged(bool flag) { return __any_sync(0xffffffffu, flag); }
-// Shared memory of one warp of a solve kernel: its groups' regions, or one
-// path's FP64 matrix, whichever is larger.
-constexpr int warp_smem(int groups_bytes, int n) {
-  return std::max(groups_bytes, (lu64_entries(n) + lu64_col_entries(n)) * 16);
+// Shared memory of one warp of a solve kernel: its groups' regions, or the
+// FP64 matrices of the paths re-solved at once, whichever is larger.
+template <int G, int R>
+__host__ __device__ constexpr int warp_smem(int groups_bytes, int n) {
+  const int mats = 32 / Resolve<G, R>::GS * (lu64_entries(n) + lu64_col_entries(n)) * 16;
+  return groups_bytes > mats ? groups_bytes : mats;
 }
 
 // One FP32 Euler-Newton step per ACTIVE path: consolidated solve, then the
@@ -650,7 +691,7 @@ solve_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __gr
   float cond;
   const bool ok = group_solve<float, 32, 1>(n, P, xE, xN, cond, sm) && fin;
   if (ok && !(cond <= (float)prm.cond_max))
-    resolve_flagged(32, true, n, n, path, path, vbase, ext, S, prm, (double2*)sm);
+    resolve_flagged<32, 1>(32, true, n, n, path, path, vbase, ext, S, prm, (double2*)sm);
   else
     update_path<float, 32, 1>(n, path, vbase, status, ok, xE, xN, S, prm);
 }
@@ -907,28 +948,25 @@ __device__ __forceinline__ bool gj_path(int n, int nmax, int64_t q, int64_t path
   update_path<float, G, R>(n, path, vbase, status, ok, wE, wN, S, prm);
   return false;
 }
-// Bytes of a warp: its groups' regions; they also hold one path's FP64 matrix.
+// Bytes of a warp's groups.
 template <int G, int R>
-__host__ __device__ constexpr int gj_warp_bytes() {
-  static_assert((32 / G) * GjLayout<G, G * R>::bytes >= (G * R * (G * R + 2) + 1 + (G * R + 3) / 4) * 16,
-                "a warp's regions hold one path's FP64 matrix");
-  return (32 / G) * GjLayout<G, G * R>::bytes;
-}
+__host__ __device__ constexpr int gj_groups_bytes() { return (32 / G) * GjLayout<G, G * R>::bytes; }
 
 template <int G, int R>
 __global__ void __launch_bounds__(kSolveThreads, R == 1 ? 6 : 4)
 gj_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
-                 const __grid_constant__ hpt_params prm) {
+                 const __grid_constant__ hpt_params prm, int ws) {
   extern __shared__ __align__(16) unsigned char smem[];
   grid_wait();
   const int64_t path = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int32_t status = path < p ? S.status[path] : -1;
   if (!__any_sync(0xffffffffu, status == HPT_PATH_ACTIVE)) return;   // warp-uniform exit
+  unsigned char* wsm = smem + (threadIdx.x / 32) * ws;
   const bool again = gj_path<G, R>(n, n, path, path, (size_t)path * n, status, ext, S, prm,
-                                   smem + (threadIdx.x / G) * GjLayout<G, G * R>::bytes);
+                                   wsm + ((threadIdx.x & 31) / G) * GjLayout<G, G * R>::bytes);
   if (any_flagged(again))
-    resolve_flagged(G, again, n, n, path, path, (size_t)path * n, ext, S, prm,
-                    (double2*)(smem + (threadIdx.x / 32) * gj_warp_bytes<G, R>()));
+    resolve_flagged<Resolve<G, R>::GS, Resolve<G, R>::RS>(G, again, n, n, path, path, (size_t)path * n, ext, S, prm,
+                                                          (double2*)wsm);
 }
 
 // The same over a position map (many systems), persistent as
@@ -937,9 +975,10 @@ gj_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __grid_
 template <int G, int R>
 __global__ void __launch_bounds__(kSolveThreads, R == 1 ? 6 : 4)
 gj_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
-                     const __grid_constant__ hpt_params prm, PathMap pm) {
+                     const __grid_constant__ hpt_params prm, PathMap pm, int ws) {
   extern __shared__ __align__(16) unsigned char smem[];
   grid_wait();
+  unsigned char* wsm = smem + (threadIdx.x / 32) * ws;
   constexpr int per_warp = 32 / G;
   const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
@@ -952,11 +991,10 @@ gj_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const __
     const int32_t status = path >= 0 ? S.status[path] : -1;
     if (!__any_sync(0xffffffffu, status == HPT_PATH_ACTIVE)) continue;   // warp-uniform skip
     const size_t vbase = status == HPT_PATH_ACTIVE ? pm_vbase(pm, path, n) : 0;
-    const bool again = gj_path<G, R>(n, pm.nmax, q, path, vbase, status, ext, S, prm,
-                                     smem + (threadIdx.x / G) * GjLayout<G, G * R>::bytes);
+    const bool again = gj_path<G, R>(n, pm.nmax, q, path, vbase, status, ext, S, prm, wsm + g * GjLayout<G, G * R>::bytes);
     if (any_flagged(again))
-      resolve_flagged(G, again, n, pm.nmax, q, path, vbase, ext, S, prm,
-                      (double2*)(smem + (threadIdx.x / 32) * gj_warp_bytes<G, R>()));
+      resolve_flagged<Resolve<G, R>::GS, Resolve<G, R>::RS>(G, again, n, pm.nmax, q, path, vbase, ext, S, prm,
+                                                            (double2*)wsm);
   }
 }
 
@@ -1006,7 +1044,9 @@ solve_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const
     const bool again = valid && ok && !(cond <= (T)prm.cond_max);
     if (valid && !again) update_path<T, G, R>(n, path, vbase, status, ok, xE, xN, S, prm);   // group-uniform
     __syncwarp();
-    if (any_flagged(again)) resolve_flagged(G, again, n, nmax, q, path, vbase, ext, S, prm, (double2*)wsm);
+    if (any_flagged(again))
+      resolve_flagged<Resolve<G, R>::GS, Resolve<G, R>::RS>(G, again, n, nmax, q, path, vbase, ext, S, prm,
+                                                            (double2*)wsm);
     __syncwarp();
   }
 }
@@ -1349,8 +1389,8 @@ cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
   constexpr int groups = (32 / G) * GroupSmem<float, G * R>::bytes;
-  const int ws = warp_smem(groups, std::min(pm.nmax, G * R)), smem = (kSolveThreads / 32) * ws;
-  cudaError_t e = allow_smem<(kSolveThreads / 32) * warp_smem(groups, G * R)>(solve_update_map_kernel<G, R>, smem);
+  const int ws = warp_smem<G, R>(groups, std::min(pm.nmax, G * R)), smem = (kSolveThreads / 32) * ws;
+  cudaError_t e = allow_smem<(kSolveThreads / 32) * warp_smem<G, R>(groups, G * R)>(solve_update_map_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
   return launch_chained(solve_update_map_kernel<G, R>, solve_grid(a.p, G), kSolveThreads, smem, st, pm.chained, a.n, a.p,
                         (const float2*)a.ext, a.st, a.prm, pm, ws);
@@ -1360,19 +1400,20 @@ cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
 // system or a position map.
 template <int G, int R>
 cudaError_t launch_gj(const StepArgs& a, cudaStream_t st) {
-  constexpr int smem = (kSolveThreads / G) * GjLayout<G, G * R>::bytes;
-  if (!a.map.list) {
-    cudaError_t e = allow_smem<smem>(gj_update_kernel<G, R>, smem);
-    if (e != cudaSuccess) return e;
-    return launch_chained(gj_update_kernel<G, R>, blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st, true, a.n,
-                          a.p, (const float2*)a.ext, a.st, a.prm);
-  }
-  cudaError_t e = allow_smem<smem>(gj_update_map_kernel<G, R>, smem);
-  if (e != cudaSuccess) return e;
+  constexpr int groups = gj_groups_bytes<G, R>(), most = (kSolveThreads / 32) * warp_smem<G, R>(groups, G * R);
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
+  const int ws = warp_smem<G, R>(groups, std::min(pm.nmax, G * R)), smem = (kSolveThreads / 32) * ws;
+  if (!a.map.list) {
+    cudaError_t e = allow_smem<most>(gj_update_kernel<G, R>, smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(gj_update_kernel<G, R>, blocks_for(a.p * G, kSolveThreads), kSolveThreads, smem, st, true, a.n,
+                          a.p, (const float2*)a.ext, a.st, a.prm, ws);
+  }
+  cudaError_t e = allow_smem<most>(gj_update_map_kernel<G, R>, smem);
+  if (e != cudaSuccess) return e;
   return launch_chained(gj_update_map_kernel<G, R>, solve_grid(a.p, G), kSolveThreads, smem, st, pm.chained, a.n, a.p,
-                        (const float2*)a.ext, a.st, a.prm, pm);
+                        (const float2*)a.ext, a.st, a.prm, pm, ws);
 }
 
 template <int G, int R>
@@ -1441,8 +1482,8 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
     e = shape == 0 ? launch_gj<8, 1>(a, st) : launch_gj<8, 2>(a, st);
   } else {
     pi = prof_begin(s, "solve_update_fp32", st);
-    const int ws = warp_smem(GroupSmem<float, 32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
-    e = allow_smem<(kSolveThreads / 32) * warp_smem(GroupSmem<float, 32>::bytes, kMaxN)>(solve_update_kernel, smem);
+    const int ws = warp_smem<32, 1>(GroupSmem<float, 32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
+    e = allow_smem<(kSolveThreads / 32) * warp_smem<32, 1>(GroupSmem<float, 32>::bytes, kMaxN)>(solve_update_kernel, smem);
     if (e != cudaSuccess) return e;
     e = launch_chained(solve_update_kernel, blocks_for(a.p, kSolveThreads / 32), kSolveThreads, smem, st, true, a.n, a.p,
                        (const float2*)a.ext, a.st, a.prm, ws);
