@@ -34,11 +34,6 @@ __device__ __forceinline__ cx<T> cscale(cx<T> a, T s) {
   return mk<T>(a.x * s, a.y * s);
 }
 template <typename T>
-__device__ __forceinline__ cx<T> cdiv(cx<T> a, cx<T> b) {
-  const T d = b.x * b.x + b.y * b.y;
-  return mk<T>((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
-}
-template <typename T>
 __device__ __forceinline__ cx<T> cmul_conj_scale(cx<T> a, cx<T> b, T r) {   // a conj(b) r
   return mk<T>((a.x * b.x + a.y * b.y) * r, (a.y * b.x - a.x * b.y) * r);
 }
@@ -60,30 +55,22 @@ __device__ __forceinline__ double t_hypot(double a, double b) { return hypot(a, 
 __device__ __forceinline__ float t_max(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double t_max(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ float t_min(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double t_min(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ float t_sqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ double t_sqrt(double a) { return sqrt(a); }
-// Reciprocal on the elimination's critical path: the approximate MUFU
-// reciprocal (at most 1 ulp off) for FP32, whose solves the Newton corrector
-// refines anyway; a correctly rounded one for FP64.
+// Reciprocal on the FP32 elimination's critical path: the approximate MUFU
+// reciprocal (at most 1 ulp off), since the Newton corrector refines the
+// solves anyway.
 __device__ __forceinline__ float t_rcp(float a) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
   return r;
 }
-__device__ __forceinline__ double t_rcp(double a) { return 1.0 / a; }
 __device__ __forceinline__ float t_abs(float a) { return fabsf(a); }
-__device__ __forceinline__ double t_abs(double a) { return fabs(a); }
 // 2^-e for m in [2^(e-1), 2^e): an exact power-of-two scale bringing m to
 // [1/2, 1), read off the exponent field (1 for zero, subnormal, inf, NaN).
 __device__ __forceinline__ float pow2_inv(float m) {
   const unsigned b = (__float_as_uint(m) >> 23) & 0xffu;
   return (b == 0u || b == 0xffu) ? 1.f : __uint_as_float((253u - min(b, 252u)) << 23);
-}
-__device__ __forceinline__ double pow2_inv(double m) {
-  const unsigned long long b = ((unsigned long long)__double_as_longlong(m) >> 52) & 0x7ffull;
-  return (b == 0ull || b == 0x7ffull) ? 1.0
-                                      : __longlong_as_double((long long)((2045ull - min(b, 2044ull)) << 52));
 }
 template <typename T>
 __device__ __forceinline__ T cabs_t(cx<T> a) {

@@ -1,5 +1,6 @@
 // FP64 solve of one path's consolidated system in shared memory, for the FP64
-// step, the polish and the adjoint.  Internal to libhpt.
+// step (affine and projective), the directions, the polish, the adjoint and the
+// mixed step's re-solves.  Internal to libhpt.
 //
 // What bounds an FP64 solve on sm_103a is the FP64 pipe, two lanes a clock
 // per SM: one warp-wide FP64 instruction takes as long as 64 issue slots,
@@ -256,9 +257,15 @@ __device__ __forceinline__ cx<double> lu64_x(int n, const double2* A, const int*
 // more of them without an entry (n = 8: 75 FP64 instructions a path with 8
 // lanes, 116 with 16, 200 with 32); below kLuWarps the chain counts (adjoint, n
 // = 8, 4,096 solutions: kernel 70 us with 32 lanes, 63 with 8, 61 with 16).
-// For n > 16 the line lies at four fifths of that (step of 2,300 paths, n = 24:
-// 195 us with 32 lanes, 162 with 16; 2,000 paths, n = 18: 121 and 96; 1,500
-// paths, n = 24: 150 and 162).
+// For n > 16 the line lies at four fifths of that, 1,946 paths (32 and 16
+// lanes, 1,500 | 1,946 paths: step at n = 24 150, 162 | 195, 162 us at 2,300;
+// whole calls at n = 18, directions 130, 132 | 155, 134, projective directions
+// 140, 141 | 168, 142, polish 148, 147 | 173, 149, adjoint 144, 153 | 169, 153;
+// at n = 24, 186, 202 | 232, 204; 200, 216 | 251, 216; 203, 216 | 250, 219;
+// 202, 223 | 248, 225).  The 16-lane blocks take twice the shared memory, and
+// past one wave of them (2,432 paths at n = 24, 1,216 at n = 31) 32 lanes are
+// faster again for a while (3,000 paths, directions at n = 24 366 and 292, at n
+// = 31 643 and 552): one line for all n is kept.
 // Shapes: 0 (8, 1), 1 (8, 2), 2 (16, 2), 3 (32, 1), 4 (16, 1), (lanes, unknowns
 // per lane).  Every shape gives the same bits.
 constexpr int64_t kLuWarps = 152 * 4 * 2;

@@ -1,6 +1,8 @@
 // Algorithm 3 (EulerNewton, Section 6) in its QR null-space form, for the
 // projective formulation (Section 2.2) and, without the y^* row, for the
-// affine one; plus the step of the projective tracker.
+// affine one; plus the step of the projective tracker.  The reflectors below
+// are the FP32 form; FP64 takes both directions from one LU solve
+// (null64_kernel).
 //
 // The consolidated matrix of one point is
 //   J = [[dH/dy, dH/dtau, H], [y^*, 0, 0]]      (N x (N+2), N = nv)
@@ -500,7 +502,7 @@ __device__ __forceinline__ void update_proj(int n, int nv, int64_t path, size_t 
 // points y (p x nv), directions to dE, dN, regularity to ok.  STEP = true:
 // one projective step of every ACTIVE path of the state.
 template <typename T, int G, int R, int CM, bool STEP>
-__global__ void __launch_bounds__(kQrThreads, (sizeof(T) == 4 && R == 3 && CM == 20) ? 3 : 1)
+__global__ void __launch_bounds__(kQrThreads, (R == 3 && CM == 20) ? 3 : 1)
 qr_kernel(int n, int nv, int proj, int64_t p, const void* __restrict__ ext, const void* __restrict__ yin,
           void* __restrict__ dE, void* __restrict__ dN, int32_t* __restrict__ okout, hpt_paths S, hpt_params prm) {
   extern __shared__ __align__(16) unsigned char smem[];

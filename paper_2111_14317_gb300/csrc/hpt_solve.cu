@@ -6,18 +6,21 @@
 // D_z H w = r, d = diag(y) w: the diag(1/y) scaling of op. 3 of Algorithm 2
 // costs n products per path here instead of n^2 in the evaluation.
 //
-// Solve mapping: a group of G lanes owns one path and every lane holds R rows
-// of [D_z H | -H_tau | -H] in registers (rows lane, lane + G, ...), n <= G R.
-// The rows are equilibrated by exact powers of two, then Gaussian elimination
-// with partial pivoting runs over a run-time column loop.  Rows are "shifted":
-// after column j is eliminated every live row moves one register to the left,
-// so the current column is always register 0 and the loop body uses static
-// register indices only.  The pivot (largest |.|^2; ties to the lowest row, as
-// LAPACK's getrf) comes from one packed integer max per butterfly level; its
-// owner writes the pivot row, relative to column j, into row j of the group's
-// shared-memory factor U, from where every lane reads it.  Back substitution
-// works column by column on U.  Two right-hand sides [-H_tau, -H] give the
-// Euler direction dE and the Newton direction dN from one factorisation.
+// Three solves.  FP64 (step, polish, adjoint, re-solve): LU in shared memory,
+// hpt_lu64.cuh.  FP32, n <= 16: Gauss-Jordan with the rows in registers
+// (gj_path).  FP32, n > 16 (group_solve): a group of G lanes owns one path and
+// every lane holds R rows of [D_z H | -H_tau | -H] in registers (rows lane,
+// lane + G, ...), n <= G R.  The rows are equilibrated by exact powers of two,
+// then Gaussian elimination with partial pivoting runs over a run-time column
+// loop.  Rows are "shifted": after column j is eliminated every live row moves
+// one register to the left, so the current column is always register 0 and the
+// loop body uses static register indices only.  The pivot (largest |.|^2; ties
+// to the lowest row, as LAPACK's getrf) comes from one packed integer max per
+// butterfly level; its owner writes the pivot row, relative to column j, into
+// row j of the group's shared-memory factor U, from where every lane reads it.
+// Back substitution works column by column on U.  Two right-hand sides
+// [-H_tau, -H] give the Euler direction dE and the Newton direction dN from one
+// factorisation, in every form.
 #include <math.h>
 
 #include <algorithm>
@@ -30,13 +33,11 @@
 namespace hpt {
 namespace {
 
-// Pivot key: |a|^2 rounded to float with the low five mantissa bits replaced
+// Pivot key: |a|^2 with the low five mantissa bits replaced
 // by (31 - row), so that one integer max picks the largest magnitude, ties to
 // the lowest row.  Rows already used as pivots get key 0.
-template <typename T>
-__device__ __forceinline__ unsigned pivot_key(T v, bool used, int row) {
+__device__ __forceinline__ unsigned pivot_key(float f, bool used, int row) {
   if (used) return 0u;
-  float f = (float)v;
   if (!(f == f)) f = 0.f;   // NaN rows stay eligible; the pivot test flags them
   return (__float_as_uint(f) & ~31u) | (unsigned)(31 - row);
 }
@@ -45,10 +46,10 @@ __device__ __forceinline__ unsigned pivot_key(T v, bool used, int row) {
 // 16-byte aligned, LD - 1 odd keeps the column reads of the back substitution
 // on distinct banks) then the column scales (NC reals), padded so that
 // consecutive groups start 8 banks apart.
-template <typename T, int NC>
+template <int NC>
 struct GroupSmem {
   static constexpr int LD = NC + 4;
-  static constexpr int raw_words = (NC * LD * 2 * (int)sizeof(T) + NC * (int)sizeof(T)) / 4;
+  static constexpr int raw_words = NC * LD * 2 + NC;
   static constexpr int words = (raw_words + 31) / 32 * 32 + 8;
   static constexpr int bytes = words * 4;
 };
@@ -57,41 +58,41 @@ constexpr int kSolveThreads = 128;
 
 // Rows of one path for a group: lane l holds rows l + G s, s < R, as
 // a[s][0..NC) plus the two right-hand sides.
-template <typename T, int G, int R>
+template <int G, int R>
 struct PathRows {
   static constexpr int NC = G * R;
-  cx<T> a[R][NC];
-  cx<T> bE[R], bN[R];
+  cx<float> a[R][NC];
+  cx<float> bE[R], bN[R];
 };
 
 
 // Loads the rows of [D_z H | -H_tau | -H] of one path; returns whether every
 // entry is finite (group-uniform).
-template <typename T, int G, int R>
+template <int G, int R>
 __device__ __forceinline__ bool load_rows(int n, int nmax, const void* ext, int64_t q, bool valid,
-                                          PathRows<T, G, R>& P) {
+                                          PathRows<G, R>& P) {
   constexpr int NC = G * R;
   const int lane = threadIdx.x & (G - 1);
-  T chk = T(0);
+  float chk = 0.f;
 #pragma unroll
   for (int s = 0; s < R; ++s) {
     const int r = lane + G * s;
     const bool have = valid && r < n;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      P.a[s][c] = mk<T>(0, 0);
+      P.a[s][c] = mk<float>(0, 0);
       if (have && c < n) {
-        P.a[s][c] = ld<T>(ext, ext_index(q, r, c, nmax));
+        P.a[s][c] = ld<float>(ext, ext_index(q, r, c, nmax));
         chk += t_abs(P.a[s][c].x) + t_abs(P.a[s][c].y);
       }
     }
-    P.bE[s] = mk<T>(0, 0);
-    P.bN[s] = mk<T>(0, 0);
+    P.bE[s] = mk<float>(0, 0);
+    P.bN[s] = mk<float>(0, 0);
     if (have) {
-      const cx<T> ht = ld<T>(ext, ext_index(q, r, n, nmax));
-      const cx<T> h = ld<T>(ext, ext_index(q, r, n + 1, nmax));
-      P.bE[s] = mk<T>(-ht.x, -ht.y);
-      P.bN[s] = mk<T>(-h.x, -h.y);
+      const cx<float> ht = ld<float>(ext, ext_index(q, r, n, nmax));
+      const cx<float> h = ld<float>(ext, ext_index(q, r, n + 1, nmax));
+      P.bE[s] = mk<float>(-ht.x, -ht.y);
+      P.bN[s] = mk<float>(-h.x, -h.y);
       chk += t_abs(P.bE[s].x) + t_abs(P.bE[s].y) + t_abs(P.bN[s].x) + t_abs(P.bN[s].y);
     }
   }
@@ -110,44 +111,39 @@ __device__ __forceinline__ bool load_rows(int n, int nmax, const void* ext, int6
 // banks).  Only paths with act set are read.  Call with every thread of the
 // block between two block barriers.
 constexpr int kStageLD = 35;
-template <typename S>
 __device__ __forceinline__ void stage_block_rows(int n, int nmax, const void* __restrict__ ext, int64_t q0, bool act,
                                                  unsigned char* smem, int region_bytes) {
   if (!act) return;   // act: path (threadIdx.x & 3) of the block is to be solved
-  typedef typename cplx_t<S>::type V;
   const int i = threadIdx.x & 3;
-  V* region = (V*)(smem + i * region_bytes);
+  float2* region = (float2*)(smem + i * region_bytes);
   const int np2 = n + 2, total = n * np2;
   for (int e = threadIdx.x >> 2; e < total; e += 32) {
     const int k = e / np2, u = e - k * np2;
-    region[k * kStageLD + u] = ((const V*)ext)[ext_index(q0 + i, k, u, nmax)];
+    region[k * kStageLD + u] = ((const float2*)ext)[ext_index(q0 + i, k, u, nmax)];
   }
 }
 
 // load_rows for a 32-lane group from its staged region (lane r = row r).
-template <typename T, typename S>
-__device__ __forceinline__ bool load_rows_staged(int n, const unsigned char* region, bool valid,
-                                                 PathRows<T, 32, 1>& P) {
-  typedef typename cplx_t<S>::type V;
-  const V* rg = (const V*)region;
+__device__ __forceinline__ bool load_rows_staged(int n, const unsigned char* region, bool valid, PathRows<32, 1>& P) {
+  const float2* rg = (const float2*)region;
   const int r = threadIdx.x & 31;
   const bool have = valid && r < n;
-  T chk = T(0);
+  float chk = 0.f;
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
-    P.a[0][c] = mk<T>(0, 0);
+    P.a[0][c] = mk<float>(0, 0);
     if (have && c < n) {
-      const V v = rg[r * kStageLD + c];
-      P.a[0][c] = mk<T>((T)v.x, (T)v.y);
+      const float2 v = rg[r * kStageLD + c];
+      P.a[0][c] = mk<float>(v.x, v.y);
       chk += t_abs(P.a[0][c].x) + t_abs(P.a[0][c].y);
     }
   }
-  P.bE[0] = mk<T>(0, 0);
-  P.bN[0] = mk<T>(0, 0);
+  P.bE[0] = mk<float>(0, 0);
+  P.bN[0] = mk<float>(0, 0);
   if (have) {
-    const V ht = rg[r * kStageLD + n], h = rg[r * kStageLD + n + 1];
-    P.bE[0] = mk<T>(-(T)ht.x, -(T)ht.y);
-    P.bN[0] = mk<T>(-(T)h.x, -(T)h.y);
+    const float2 ht = rg[r * kStageLD + n], h = rg[r * kStageLD + n + 1];
+    P.bE[0] = mk<float>(-ht.x, -ht.y);
+    P.bN[0] = mk<float>(-h.x, -h.y);
     chk += t_abs(P.bE[0].x) + t_abs(P.bE[0].y) + t_abs(P.bN[0].x) + t_abs(P.bN[0].y);
   }
   __syncwarp();   // every row is in registers before the solve writes U over the region
@@ -159,21 +155,21 @@ __device__ __forceinline__ bool load_rows_staged(int n, const unsigned char* reg
 // finite; cond receives max |u_jj| / min |u_jj|.  On return lane l holds
 // solution components l + G s in xE[s], xN[s].  sm is the group's shared
 // memory (GroupSmem).
-template <typename T, int G, int R>
-__device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (&xE)[R], cx<T> (&xN)[R], T& cond,
-                            unsigned char* sm) {
-  constexpr int NC = G * R, LD = GroupSmem<T, NC>::LD;
-  cx<T>* U = (cx<T>*)sm;
-  T* dcol = (T*)(sm + NC * LD * sizeof(cx<T>));
+template <int G, int R>
+__device__ __forceinline__ bool group_solve(int n, PathRows<G, R>& P, cx<float> (&xE)[R], cx<float> (&xN)[R],
+                                            float& cond, unsigned char* sm) {
+  constexpr int NC = G * R, LD = GroupSmem<NC>::LD;
+  cx<float>* U = (cx<float>*)sm;
+  float* dcol = (float*)(sm + NC * LD * sizeof(cx<float>));
   const int lane = threadIdx.x & (G - 1);
 
   // equilibration: rows, then columns, by exact powers of two
 #pragma unroll
   for (int s = 0; s < R; ++s) {
-    T m = T(0);
+    float m = 0.f;
 #pragma unroll
     for (int c = 0; c < NC; ++c) m = t_max(m, cmag(P.a[s][c]));
-    const T dr = pow2_inv(m);
+    const float dr = pow2_inv(m);
 #pragma unroll
     for (int c = 0; c < NC; ++c) P.a[s][c] = cscale(P.a[s][c], dr);
     P.bE[s] = cscale(P.bE[s], dr);
@@ -182,12 +178,12 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     if (c < n) {
-      T m = T(0);
+      float m = 0.f;
 #pragma unroll
       for (int s = 0; s < R; ++s) m = t_max(m, cmag(P.a[s][c]));
 #pragma unroll
       for (int o = G / 2; o > 0; o >>= 1) m = t_max(m, __shfl_xor_sync(0xffffffffu, m, o, G));
-      const T d = pow2_inv(m);
+      const float d = pow2_inv(m);
 #pragma unroll
       for (int s = 0; s < R; ++s) P.a[s][c] = cscale(P.a[s][c], d);
       if (lane == 0) dcol[c] = d;
@@ -198,12 +194,12 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
 #pragma unroll
   for (int s = 0; s < R; ++s) used[s] = lane + G * s >= n;
   bool ok = true;
-  T pmax = 0, pmin = 0;   // extreme |u_jj|^2
+  float pmax = 0, pmin = 0;   // extreme |u_jj|^2
 #pragma unroll 1
   for (int j = 0; j < n; ++j) {
     unsigned key = 0u;
 #pragma unroll
-    for (int s = 0; s < R; ++s) key = max(key, pivot_key<T>(abs2(P.a[s][0]), used[s], lane + G * s));
+    for (int s = 0; s < R; ++s) key = max(key, pivot_key(abs2(P.a[s][0]), used[s], lane + G * s));
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o, G));
     const int br = 31 - (int)(key & 31u);
@@ -213,12 +209,12 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
       const int bs = br / G;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        cx<T> v = P.a[0][c];
+        cx<float> v = P.a[0][c];
 #pragma unroll
         for (int s = 1; s < R; ++s) v = (bs == s) ? P.a[s][c] : v;
         U[j * LD + c] = v;
       }
-      cx<T> e = P.bE[0], f = P.bN[0];
+      cx<float> e = P.bE[0], f = P.bN[0];
 #pragma unroll
       for (int s = 1; s < R; ++s) {
         e = (bs == s) ? P.bE[s] : e;
@@ -230,17 +226,17 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
       for (int s = 0; s < R; ++s) used[s] = used[s] || (bs == s);
     }
     __syncwarp();
-    const cx<T> pj = U[j * LD];
-    const T p2 = abs2(pj);
-    if (!(p2 > T(0)) || !isfinite(p2)) ok = false;
+    const cx<float> pj = U[j * LD];
+    const float p2 = abs2(pj);
+    if (!(p2 > 0.f) || !isfinite(p2)) ok = false;
     pmax = j == 0 ? p2 : t_max(pmax, p2);
     pmin = j == 0 ? p2 : t_min(pmin, p2);
-    const T rp = t_rcp(p2);   // one reciprocal per pivot, shared by all rows
+    const float rp = t_rcp(p2);   // one reciprocal per pivot, shared by all rows
     // multipliers; rows already used get 0, so the unpredicated update below
     // only shifts them (their values are no longer read)
-    cx<T> l[R];
+    cx<float> l[R];
 #pragma unroll
-    for (int s = 0; s < R; ++s) l[s] = used[s] ? mk<T>(0, 0) : cmul_conj_scale(P.a[s][0], pj, rp);
+    for (int s = 0; s < R; ++s) l[s] = used[s] ? mk<float>(0, 0) : cmul_conj_scale(P.a[s][0], pj, rp);
     // shifted update: a[c-1] = a[c] - l u_{j, j+c} over the live width, in
     // chunks of four columns behind one warp-uniform branch each (the
     // columns of the last chunk beyond the live width are updated too; they
@@ -252,14 +248,14 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
 #pragma unroll
         for (int c = c0; c < c0 + 4; ++c) {
           if (c < NC) {
-            const cx<T> u = U[j * LD + c];
+            const cx<float> u = U[j * LD + c];
 #pragma unroll
             for (int s = 0; s < R; ++s) P.a[s][c - 1] = csub_mul(P.a[s][c], l[s], u);
           }
         }
       }
     }
-    const cx<T> uE = U[j * LD + NC], uN = U[j * LD + NC + 1];
+    const cx<float> uE = U[j * LD + NC], uN = U[j * LD + NC + 1];
 #pragma unroll
     for (int s = 0; s < R; ++s) {
       P.bE[s] = csub_mul(P.bE[s], l[s], uE);
@@ -269,33 +265,33 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
   __syncwarp();
   // back substitution on U (row i holds u_{i, i+c} at c, then the two
   // right-hand sides); lane l carries the right-hand sides of rows l + G s
-  cx<T> rE[R], rN[R];
+  cx<float> rE[R], rN[R];
 #pragma unroll
   for (int s = 0; s < R; ++s) {
     const int i = lane + G * s;
-    rE[s] = i < n ? U[i * LD + NC] : mk<T>(0, 0);
-    rN[s] = i < n ? U[i * LD + NC + 1] : mk<T>(0, 0);
-    xE[s] = mk<T>(0, 0);
-    xN[s] = mk<T>(0, 0);
+    rE[s] = i < n ? U[i * LD + NC] : mk<float>(0, 0);
+    rN[s] = i < n ? U[i * LD + NC + 1] : mk<float>(0, 0);
+    xE[s] = mk<float>(0, 0);
+    xN[s] = mk<float>(0, 0);
   }
 #pragma unroll 1
   for (int j = n - 1; j >= 0; --j) {
-    const cx<T> ujj = U[j * LD];
+    const cx<float> ujj = U[j * LD];
     const int js = j / G;
-    cx<T> vE = rE[0], vN = rN[0];
+    cx<float> vE = rE[0], vN = rN[0];
 #pragma unroll
     for (int s = 1; s < R; ++s)
       if (s == js) { vE = rE[s]; vN = rN[s]; }
-    vE = shfl<T, G>(vE, j & (G - 1));
-    vN = shfl<T, G>(vN, j & (G - 1));
-    const T ru = t_rcp(abs2(ujj));
-    const cx<T> xe = cmul_conj_scale(vE, ujj, ru), xn = cmul_conj_scale(vN, ujj, ru);
+    vE = shfl<float, G>(vE, j & (G - 1));
+    vN = shfl<float, G>(vN, j & (G - 1));
+    const float ru = t_rcp(abs2(ujj));
+    const cx<float> xe = cmul_conj_scale(vE, ujj, ru), xn = cmul_conj_scale(vN, ujj, ru);
 #pragma unroll
     for (int s = 0; s < R; ++s) {
       const int i = lane + G * s;
       if (i == j) { xE[s] = xe; xN[s] = xn; }
       if (i < j) {
-        const cx<T> u = U[i * LD + (j - i)];
+        const cx<float> u = U[i * LD + (j - i)];
         rE[s] = csub_mul(rE[s], u, xe);
         rN[s] = csub_mul(rN[s], u, xn);
       }
@@ -305,13 +301,13 @@ __device__ __forceinline__ bool group_solve(int n, PathRows<T, G, R>& P, cx<T> (
   for (int s = 0; s < R; ++s) {
     const int i = lane + G * s;
     if (i < n) {
-      const T d = dcol[i];
+      const float d = dcol[i];
       xE[s] = cscale(xE[s], d);
       xN[s] = cscale(xN[s], d);
     }
   }
   __syncwarp();   // the group's shared memory is reused by its next solve
-  cond = pmin > T(0) ? t_sqrt(pmax / pmin) : T(INFINITY);
+  cond = pmin > 0.f ? t_sqrt(pmax / pmin) : INFINITY;
   return ok;
 }
 
@@ -681,15 +677,15 @@ solve_update_kernel(int n, int64_t p, const float2* __restrict__ ext, const __gr
   unsigned char* sm = smem + (threadIdx.x / 32) * ws;
   const int64_t q0 = (int64_t)blockIdx.x * (kSolveThreads / 32);
   const int64_t qi = q0 + (threadIdx.x & 3);
-  stage_block_rows<float>(n, n, ext, q0, qi < p && S.status[qi] == HPT_PATH_ACTIVE, smem, ws);
+  stage_block_rows(n, n, ext, q0, qi < p && S.status[qi] == HPT_PATH_ACTIVE, smem, ws);
   __syncthreads();
   if (!valid) return;   // warp-uniform
   const size_t vbase = (size_t)path * n;
-  PathRows<float, 32, 1> P;
-  const bool fin = load_rows_staged<float, float>(n, sm, valid, P);
+  PathRows<32, 1> P;
+  const bool fin = load_rows_staged(n, sm, valid, P);
   cx<float> xE[1], xN[1];
   float cond;
-  const bool ok = group_solve<float, 32, 1>(n, P, xE, xN, cond, sm) && fin;
+  const bool ok = group_solve<32, 1>(n, P, xE, xN, cond, sm) && fin;
   if (ok && !(cond <= (float)prm.cond_max))
     resolve_flagged<32, 1>(32, true, n, n, path, path, vbase, ext, S, prm, (double2*)sm);
   else
@@ -838,7 +834,7 @@ __device__ __forceinline__ bool gj_path(int n, int nmax, int64_t q, int64_t path
 #pragma unroll
     for (int s = 0; s < R; ++s) {
       const float2 v = upk2(a[s][0]);
-      key = max(key, pivot_key<float>(v.x * v.x + v.y * v.y, used[s], lane + G * s));
+      key = max(key, pivot_key(v.x * v.x + v.y * v.y, used[s], lane + G * s));
     }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o, G));
@@ -1005,7 +1001,6 @@ template <int G, int R>
 __global__ void __launch_bounds__(kSolveThreads)
 solve_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const __grid_constant__ hpt_paths S,
                         const __grid_constant__ hpt_params prm, PathMap pm, int ws) {
-  typedef float T;
   extern __shared__ __align__(16) unsigned char smem[];
   grid_wait();
   constexpr int per_warp = 32 / G;
@@ -1013,7 +1008,7 @@ solve_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const
   const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
   const int g = (threadIdx.x & 31) / G;
   unsigned char* wsm = smem + (threadIdx.x / 32) * ws;
-  unsigned char* sm = wsm + g * GroupSmem<T, G * R>::bytes;
+  unsigned char* sm = wsm + g * GroupSmem<G * R>::bytes;
   const int64_t npos = pm_count(pm, p);
   const int nmax = pm.nmax;
   // with 32-lane groups the block's four warps take consecutive positions of
@@ -1029,20 +1024,20 @@ solve_update_map_kernel(int n0, int64_t p, const float2* __restrict__ ext, const
       const int64_t q0 = base - (threadIdx.x >> 5);
       const int64_t pi = pm_path(pm, q0 + (threadIdx.x & 3));
       __syncthreads();   // the previous iteration's solves are done with the regions
-      stage_block_rows<T>(n, nmax, ext, q0, pi >= 0 && S.status[pi] == HPT_PATH_ACTIVE, smem, ws);
+      stage_block_rows(n, nmax, ext, q0, pi >= 0 && S.status[pi] == HPT_PATH_ACTIVE, smem, ws);
       __syncthreads();
     }
     if (!__any_sync(0xffffffffu, valid)) continue;   // warp-uniform skip
     const size_t vbase = valid ? pm_vbase(pm, path, n) : 0;
-    PathRows<T, G, R> P;
+    PathRows<G, R> P;
     bool fin;
-    if constexpr (G == 32) fin = load_rows_staged<T, T>(n, sm, valid, P);
-    else fin = load_rows<T, G, R>(n, nmax, ext, q, valid, P);
-    cx<T> xE[R], xN[R];
-    T cond;
-    const bool ok = group_solve<T, G, R>(n, P, xE, xN, cond, sm) && fin;
-    const bool again = valid && ok && !(cond <= (T)prm.cond_max);
-    if (valid && !again) update_path<T, G, R>(n, path, vbase, status, ok, xE, xN, S, prm);   // group-uniform
+    if constexpr (G == 32) fin = load_rows_staged(n, sm, valid, P);
+    else fin = load_rows<G, R>(n, nmax, ext, q, valid, P);
+    cx<float> xE[R], xN[R];
+    float cond;
+    const bool ok = group_solve<G, R>(n, P, xE, xN, cond, sm) && fin;
+    const bool again = valid && ok && !(cond <= (float)prm.cond_max);
+    if (valid && !again) update_path<float, G, R>(n, path, vbase, status, ok, xE, xN, S, prm);   // group-uniform
     __syncwarp();
     if (any_flagged(again))
       resolve_flagged<Resolve<G, R>::GS, Resolve<G, R>::RS>(G, again, n, nmax, q, path, vbase, ext, S, prm,
@@ -1388,7 +1383,7 @@ template <int G, int R>
 cudaError_t launch_solve_map(const StepArgs& a, cudaStream_t st) {
   PathMap pm = a.map;
   if (!pm.nmax) pm.nmax = a.n;
-  constexpr int groups = (32 / G) * GroupSmem<float, G * R>::bytes;
+  constexpr int groups = (32 / G) * GroupSmem<G * R>::bytes;
   const int ws = warp_smem<G, R>(groups, std::min(pm.nmax, G * R)), smem = (kSolveThreads / 32) * ws;
   cudaError_t e = allow_smem<(kSolveThreads / 32) * warp_smem<G, R>(groups, G * R)>(solve_update_map_kernel<G, R>, smem);
   if (e != cudaSuccess) return e;
@@ -1482,8 +1477,8 @@ cudaError_t launch_solve_update(hpt_system s, const StepArgs& a, cudaStream_t st
     e = shape == 0 ? launch_gj<8, 1>(a, st) : launch_gj<8, 2>(a, st);
   } else {
     pi = prof_begin(s, "solve_update_fp32", st);
-    const int ws = warp_smem<32, 1>(GroupSmem<float, 32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
-    e = allow_smem<(kSolveThreads / 32) * warp_smem<32, 1>(GroupSmem<float, 32>::bytes, kMaxN)>(solve_update_kernel, smem);
+    const int ws = warp_smem<32, 1>(GroupSmem<32>::bytes, a.n), smem = (kSolveThreads / 32) * ws;
+    e = allow_smem<(kSolveThreads / 32) * warp_smem<32, 1>(GroupSmem<32>::bytes, kMaxN)>(solve_update_kernel, smem);
     if (e != cudaSuccess) return e;
     e = launch_chained(solve_update_kernel, blocks_for(a.p, kSolveThreads / 32), kSolveThreads, smem, st, true, a.n, a.p,
                        (const float2*)a.ext, a.st, a.prm, ws);
