@@ -728,9 +728,6 @@ def step_roofline(mx, peaks, peak_kind, sms):
                                                  f"{MUFU_SINCOS_PER_CLK}/clk/SM",
                         "tensor": {"achieved": gemm / avg / 1e12, "peak": bf16, "unit": "TFLOP/s",
                                    "frac": gemm / avg / 1e12 / bf16, "peak_source": src}})
-        elif name.startswith("redo"):
-            # re-solves a device-side list of a few paths: no per-path figure
-            rec.update({"bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None})
         else:
             fl = (FLOP_LU + FLOP_SOLVE) * ppl
             ach = fl / avg / 1e12

@@ -18,8 +18,10 @@
 // (ACM TOMS 16, 1990) with 128 entries, the angle by the addition theorem of
 // atan with tan(alpha_i) = i/32.  The tables are computed by the compiler
 // from Taylor series, repeated squaring and Euler's series, in 128-bit
-// integers.  Errors: about 2^-59 absolute in log2|y| and in the fractions,
-// 2^-62 in the angle (the tests compare with long double).
+// integers.  Largest errors over a million random arguments, against 113 bits:
+// 2^-58.5 in log2|y|, 2^-59.7 revolution in the angle, 2^-57.7 in cos and sin,
+// 2^-57.2 in exp2 (of values up to 2); what is exact: phases of whole quarter
+// turns (points on the axes) and their cos and sin.
 //
 // Qn below means a fixed-point number with n fraction bits.
 #pragma once
